@@ -239,10 +239,11 @@ struct Carve {
 static size_t carve(const eco_config *c, const Layout &L, uint8_t *base, Dev *d, EnvDesc **env_dev) {
   Carve k;
   k.base = base;
-  long long cells = 0, slots = 0;
+  long long cells = 0, slots = 0, ctiles = 0;
   for (int e = 0; e < c->n_envs; ++e) {
     cells += (long long)c->env_side[e] * c->env_side[e];
     slots += c->env_slots[e];
+    ctiles += place_tiles(c->env_side[e]);
   }
   const int E = c->n_envs;
   Dev &D = *d;
@@ -295,8 +296,10 @@ static size_t carve(const eco_config *c, const Layout &L, uint8_t *base, Dev *d,
   D.step = k.take<long long>(1);
   D.alive_at_step = k.take<int32_t>(kAliveRing);
   D.hist = k.take<uint32_t>((size_t)E * 65536);
-  D.place_prefix = k.take<unsigned long long>(E);
+  D.place_key = k.take<unsigned long long>(E);
   D.place_remaining = k.take<int32_t>(E);
+  D.place_tile_count = (int)ctiles;
+  D.place_tiles = k.take<int32_t>(ctiles);
   D.hp = k.take<int32_t>(slots);
   D.age = k.take<int32_t>(slots);
   D.res = k.take<int32_t>(cells);
@@ -417,7 +420,7 @@ extern "C" int eco_create(const eco_config *cfg, void *dev_workspace, size_t byt
   h->ws = reinterpret_cast<uint8_t *>(dev_workspace);
   h->ws_bytes = bytes;
   carve(cfg, h->L, h->ws, &h->d, &h->env_dev);
-  int so = 0, co = 0;
+  int so = 0, co = 0, to = 0;
   for (int e = 0; e < cfg->n_envs; ++e) {
     EnvDesc ed;
     ed.side = cfg->env_side[e];
@@ -426,6 +429,8 @@ extern "C" int eco_create(const eco_config *cfg, void *dev_workspace, size_t byt
     ed.cell_off = co;
     ed.init_alive = cfg->env_init_alive[e];
     ed.seed = cfg->env_seed[e];
+    ed.ctile_off = to;
+    to += place_tiles(ed.side);
     h->env_host.push_back(ed);
     so += ed.n_slots;
     co += ed.side * ed.side;

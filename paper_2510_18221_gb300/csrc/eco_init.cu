@@ -1,17 +1,16 @@
 // eco_init.cu -- reset of every environment (Sec. 3.2: grid world with
-// randomly distributed resources and a founding population; Sec. 3.3:
-// Kaiming-style initial weights, zero biases) and re-derivation of the
-// streamed BF16 / FP8 weight copy from the FP32 masters.
+// randomly distributed resources and a founding population) and the recount
+// of the statistics after a state write.  The founders' weights are drawn in
+// eco_params.cu.
 //
 // Founders: the K non-wall cells with the smallest 64-bit keys
 // (PLACE draw << 32 | local cell) -- all keys are distinct -- found by a
-// four-round radix select on 16-bit digits (one histogram pass over the
-// cells per round), then numbered in ascending cell order by a block scan.
+// radix select on the draw's two 16-bit digits (a histogram pass over the
+// cells per digit, the first one inside the pass that fills the cells), a
+// rank among the cells that share the last founder's draw, then a two-pass
+// tiled scan that numbers the founders in ascending cell order.
 #include "eco_internal.cuh"
 #include "eco_kernels.h"
-
-#include <cuda_bf16.h>
-#include <cuda_fp8.h>
 
 namespace eco {
 
@@ -20,55 +19,122 @@ __device__ __forceinline__ unsigned long long place_key(const EnvDesc &ed, int l
   return ((unsigned long long)word_of(r, local_cell & 3) << 32) | (unsigned long long)(uint32_t)local_cell;
 }
 
-// Walls, food, empty occupancy, cleared claims.  Paper rules: a food cell
-// holds one bite, e_food energy.
-__global__ void k_init_cells(Dev d, Rules R) {
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < d.total_cells; c += gridDim.x * blockDim.x) {
-    const int e = env_of_cell(d.env, d.n_envs, c);
-    const EnvDesc ed = d.env[e];
-    const int lc = c - ed.cell_off;
-    const U4 rw = philox((uint32_t)(lc >> 2), 0u, 0u, 0u, ed.seed, S_WALL);
-    const bool wall = word_of(rw, lc & 3) < R.thr_wall;
-    const U4 rf = philox((uint32_t)(lc >> 2), 0u, 0u, 0u, ed.seed, S_FOOD_INIT);
-    const bool food = !wall && word_of(rf, lc & 3) < R.thr_food;
-    d.cellf[c] = (uint8_t)((wall ? CELL_WALL : 0u) | (food ? CELL_FOOD : 0u));
-    d.res[c] = (R.rules != RULES_SIMPLE && food) ? R.e_food : 0;
-    d.occ[c] = -1;
-    // terrain rules: water fills the cells whose rock lies below sea level;
-    // a Bernoulli(biomass_density) site (stream BIOMASS) holds b_site
-    int water = 0, bio = 0;
-    if (R.rules == RULES_TERRAIN && !wall) {
-      const int rk = d.rock[c];
-      if (rk < R.sea_level) water = R.sea_level - rk;
-      const U4 rb = philox((uint32_t)(lc >> 2), 0u, 0u, 0u, ed.seed, S_BIOMASS);
-      if (word_of(rb, lc & 3) < R.thr_bio) bio = R.b_site;
-    }
-    d.water[c] = water;
-    d.bio[c] = bio;
-    d.photo[c] = 0u;
-    d.flow[c] = 0u;
-    d.claim_move[c] = 0ull;
-    d.cnt_move[c] = 0u;
-    d.claim_birth[c] = 0ull;
-    d.att_cell[c] = 0ull;
+// Walls, food, empty occupancy, cleared claims (paper rules: a food cell
+// holds one bite, e_food energy), the per-slot agent fields (founders get
+// alive / facing / energy here; their cells come from the placement below)
+// and the first digit's placement histogram.
+//
+// Bound by the writes, 53 bytes per cell: four cells per thread share each
+// Philox block and go out as 16-byte stores.  The counts of food, water and
+// biomass are summed here, per CTA, into the step's (zeroed) records, and
+// k_place_find<0> turns them into the initial statistics.
+__device__ __forceinline__ int env_of_slot(const EnvDesc *env, int n_envs, int slot) {
+  int lo = 0, hi = n_envs - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (env[mid].slot_off <= slot)
+      lo = mid;
+    else
+      hi = mid - 1;
   }
+  return lo;
 }
 
-// Per-slot agent fields (founders get alive / facing / energy here; their
-// cells come from the placement below).
-__global__ void k_init_agents(Dev d, Rules R) {
-  for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < d.total_slots; s += gridDim.x * blockDim.x) {
-    int e = 0;
-    while (e + 1 < d.n_envs && d.env[e + 1].slot_off <= s) ++e;
-    const EnvDesc ed = d.env[e];
-    const int ls = s - ed.slot_off;
-    const bool founder = ls < ed.init_alive;
-    d.env_of[s] = (uint16_t)e;
+__global__ void __launch_bounds__(256) k_reset_world(Dev d, Rules R) {
+  const int g0 = blockIdx.x * blockDim.x + threadIdx.x, gs = gridDim.x * blockDim.x;
+  const bool terrain = R.rules == RULES_TERRAIN;
+  long long sum[3] = {0, 0, 0};  // food, water, biomass of environment e
+  int e = -1;
+  EnvDesc ed = d.env[0];
+  const int stat[3] = {ST_FOOD_TOTAL, ST_WATER_CELLS, ST_BIO_CELLS};
+  auto flush = [&]() {
+    for (int k = 0; k < 3; ++k)
+      if (e >= 0 && sum[k])
+        atomicAdd((unsigned long long *)&d.stats_step[e * N_ST + stat[k]], (unsigned long long)sum[k]);
+    sum[0] = sum[1] = sum[2] = 0;
+  };
+  for (int g = g0; g < (d.total_cells >> 2); g += gs) {
+    const int c0 = g << 2;
+    if (e < 0 || (e + 1 < d.n_envs && d.env[e + 1].cell_off <= c0)) {
+      flush();
+      e = env_of_cell(d.env, d.n_envs, c0);
+      ed = d.env[e];
+    }
+    const uint32_t blk = (uint32_t)((c0 - ed.cell_off) >> 2);
+    const U4 rw = philox(blk, 0u, 0u, 0u, ed.seed, S_WALL);
+    const U4 rf = philox(blk, 0u, 0u, 0u, ed.seed, S_FOOD_INIT);
+    const U4 rp = philox(blk, 0u, 0u, 0u, ed.seed, S_PLACE);
+    U4 rb = {0u, 0u, 0u, 0u};
+    int4 rk = make_int4(0, 0, 0, 0);
+    if (terrain) {
+      rb = philox(blk, 0u, 0u, 0u, ed.seed, S_BIOMASS);
+      rk = reinterpret_cast<const int4 *>(d.rock)[g];
+    }
+    const int rkv[4] = {rk.x, rk.y, rk.z, rk.w};
+    uint8_t cf[4];
+    int res[4], water[4], bio[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const bool wall = word_of(rw, k) < R.thr_wall;
+      const bool food = !wall && word_of(rf, k) < R.thr_food;
+      cf[k] = (uint8_t)((wall ? CELL_WALL : 0u) | (food ? CELL_FOOD : 0u));
+      res[k] = (R.rules != RULES_SIMPLE && food) ? R.e_food : 0;
+      // terrain rules: water fills the cells whose rock lies below sea level;
+      // a Bernoulli(biomass_density) site (stream BIOMASS) holds b_site
+      water[k] = (terrain && !wall && rkv[k] < R.sea_level) ? R.sea_level - rkv[k] : 0;
+      bio[k] = (terrain && !wall && word_of(rb, k) < R.thr_bio) ? R.b_site : 0;
+      sum[0] += food ? 1 : 0;
+      sum[1] += water[k];
+      sum[2] += bio[k];
+      if (!wall && ed.init_alive > 0) atomicAdd(&d.hist[(size_t)e * 65536 + (word_of(rp, k) >> 16)], 1u);
+    }
+    const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+    reinterpret_cast<uchar4 *>(d.cellf)[g] = make_uchar4(cf[0], cf[1], cf[2], cf[3]);
+    reinterpret_cast<int4 *>(d.res)[g] = make_int4(res[0], res[1], res[2], res[3]);
+    reinterpret_cast<int4 *>(d.occ)[g] = make_int4(-1, -1, -1, -1);
+    reinterpret_cast<int4 *>(d.water)[g] = make_int4(water[0], water[1], water[2], water[3]);
+    reinterpret_cast<int4 *>(d.bio)[g] = make_int4(bio[0], bio[1], bio[2], bio[3]);
+    reinterpret_cast<uint4 *>(d.photo)[g] = z;
+    reinterpret_cast<uint4 *>(d.flow)[g] = z;
+    reinterpret_cast<uint4 *>(d.cnt_move)[g] = z;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      reinterpret_cast<uint4 *>(d.claim_move)[2 * g + k] = z;
+      reinterpret_cast<uint4 *>(d.claim_birth)[2 * g + k] = z;
+      reinterpret_cast<uint4 *>(d.att_cell)[2 * g + k] = z;
+    }
+  }
+  // one addition per CTA and count when its threads ended in one environment
+  __shared__ int s_e;
+  __shared__ unsigned long long s_sum[3];
+  if (threadIdx.x == 0) s_e = e;
+  if (threadIdx.x < 3) s_sum[threadIdx.x] = 0ull;
+  __syncthreads();
+  if (__syncthreads_and(e == s_e || e < 0)) {
+    for (int k = 0; k < 3; ++k) {
+      long long v = sum[k];
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
+      if ((threadIdx.x & 31) == 0 && v) atomicAdd(&s_sum[k], (unsigned long long)v);
+    }
+    __syncthreads();
+    if (threadIdx.x < 3 && s_e >= 0 && s_sum[threadIdx.x])
+      atomicAdd((unsigned long long *)&d.stats_step[s_e * N_ST + stat[threadIdx.x]], s_sum[threadIdx.x]);
+  } else {
+    flush();
+  }
+
+  for (int s = g0; s < d.total_slots; s += gs) {
+    const int es = env_of_slot(d.env, d.n_envs, s);
+    const EnvDesc eds = d.env[es];
+    const int ls = s - eds.slot_off;
+    const bool founder = ls < eds.init_alive;
+    d.env_of[s] = (uint16_t)es;
     d.alive[s] = founder ? 1 : 0;
     d.pos[s] = 0;
     uint8_t f = 0;
     if (founder) {
-      const U4 r = philox((uint32_t)(ls >> 2), 0u, 0u, 0u, ed.seed, S_FACING_INIT);
+      const U4 r = philox((uint32_t)(ls >> 2), 0u, 0u, 0u, eds.seed, S_FACING_INIT);
       f = (uint8_t)(word_of(r, ls & 3) >> 30);
     }
     d.facing[s] = f;
@@ -79,13 +145,13 @@ __global__ void k_init_agents(Dev d, Rules R) {
     d.tgt[s] = -1;
     d.gain[s] = 0;
     d.hp[s] = (founder && R.rules != RULES_SIMPLE) ? R.hp_max : 0;
-    d.a_water[s] = (founder && R.rules == RULES_TERRAIN) ? R.w_init : 0;
-    d.a_bio[s] = (founder && R.rules == RULES_TERRAIN) ? R.b_body : 0;
+    d.a_water[s] = (founder && terrain) ? R.w_init : 0;
+    d.a_bio[s] = (founder && terrain) ? R.b_body : 0;
     d.age[s] = 0;
     // colour trait (Sec. 3.3): three uniforms of COLOUR at counter (slot, 0, 0, 0)
     float4 col = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (founder) {
-      const U4 r = philox((uint32_t)ls, 0u, 0u, 0u, ed.seed, S_COLOUR);
+      const U4 r = philox((uint32_t)ls, 0u, 0u, 0u, eds.seed, S_COLOUR);
       col = make_float4(uniform01(r.x), uniform01(r.y), uniform01(r.z), 0.0f);
     }
     d.colour[s] = col;
@@ -105,200 +171,37 @@ __device__ long long block_sum_ll(long long v, unsigned long long *acc) {
   return total;
 }
 
-// Radix-select round: histogram of the 16-bit digit at `shift` among the
-// non-wall cells whose higher digits equal the prefix found so far.
-__global__ void k_place_hist(Dev d, int shift) {
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < d.total_cells; c += gridDim.x * blockDim.x) {
-    if (d.cellf[c] & CELL_WALL) continue;
-    const int e = env_of_cell(d.env, d.n_envs, c);
+// Second digit: histogram of the draw's low half among the non-wall cells
+// whose high half is the digit found first.
+__global__ void __launch_bounds__(256) k_place_hist(Dev d) {
+  const int gs = gridDim.x * blockDim.x;
+  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < (d.total_cells >> 2); g += gs) {
+    const int c0 = g << 2;
+    const int e = env_of_cell(d.env, d.n_envs, c0);
     const EnvDesc ed = d.env[e];
     if (ed.init_alive == 0) continue;
-    const unsigned long long key = place_key(ed, c - ed.cell_off);
-    if (shift < 48 && (key >> (shift + 16)) != d.place_prefix[e]) continue;
-    atomicAdd(&d.hist[(size_t)e * 65536 + ((key >> shift) & 0xFFFFull)], 1u);
-  }
-}
-
-// One CTA per environment: find the bin holding the remaining-th smallest
-// key, extend the prefix, clear the histogram.  A missing bin (fewer than K
-// non-wall cells) sets the status word.
-__global__ void __launch_bounds__(1024) k_place_find(Dev d) {
-  __shared__ int sh[33];
-  __shared__ int found_bin, found_before;
-  const int e = blockIdx.x;
-  uint32_t *h = d.hist + (size_t)e * 65536;
-  const int remaining = d.place_remaining[e];
-  if (d.env[e].init_alive == 0) return;
-  const int per = 65536 / blockDim.x;  // 64 bins per thread
-  const int beg = threadIdx.x * per;
-  int cnt = 0;
-  for (int i = 0; i < per; ++i) cnt += (int)h[beg + i];
-  int total;
-  int before = block_exclusive_scan(cnt, &total, sh);
-  if (threadIdx.x == 0) {
-    found_bin = -1;
-    found_before = 0;
-  }
-  __syncthreads();
-  if (before < remaining && before + cnt >= remaining) {
-    int run = before;
-    for (int i = 0; i < per; ++i) {
-      const int c = (int)h[beg + i];
-      if (run + c >= remaining) {
-        found_bin = beg + i;
-        found_before = run;
-        break;
-      }
-      run += c;
-    }
-  }
-  __syncthreads();
-  for (int i = 0; i < per; ++i) h[beg + i] = 0u;
-  if (threadIdx.x == 0) {
-    if (found_bin < 0) {
-      atomicOr(&d.counters[CNT_STATUS], 1);
-    } else {
-      d.place_prefix[e] = (d.place_prefix[e] << 16) | (unsigned long long)found_bin;
-      d.place_remaining[e] = remaining - found_before;
-    }
-  }
-}
-
-// One CTA per environment: founders are the non-wall cells with key <= the
-// selected threshold; slot = rank in ascending cell order.
-__global__ void __launch_bounds__(1024) k_place_assign(Dev d) {
-  __shared__ int sh[33];
-  const int e = blockIdx.x;
-  const EnvDesc ed = d.env[e];
-  if (ed.init_alive == 0) return;
-  const unsigned long long thr = d.place_prefix[e];
-  const int n = ed.side * ed.side;
-  const int per = (n + blockDim.x - 1) / blockDim.x;
-  const int beg = min(n, (int)threadIdx.x * per), end = min(n, beg + per);
-  int cnt = 0;
-  for (int c = beg; c < end; ++c)
-    if (!(d.cellf[ed.cell_off + c] & CELL_WALL) && place_key(ed, c) <= thr) ++cnt;
-  int total;
-  int off = block_exclusive_scan(cnt, &total, sh);
-  for (int c = beg; c < end; ++c) {
-    const int gc = ed.cell_off + c;
-    if (!(d.cellf[gc] & CELL_WALL) && place_key(ed, c) <= thr) {
-      // the guard only matters when the select failed (status already set)
-      if (off < ed.init_alive) {
-        const int slot = ed.slot_off + off;
-        d.pos[slot] = c;
-        d.occ[gc] = slot;
-        d.cellf[gc] |= (uint8_t)CELL_AGENT;
-      }
-      ++off;
-    }
-  }
-  if (threadIdx.x == 0 && total != ed.init_alive) atomicOr(&d.counters[CNT_STATUS], 2);
-}
-
-// Founders' weights (Sec. 3.3: Kaiming initialisation, zero biases): weight
-// p = N(0,1) * sqrt(gain / fan_in) from stream W_INIT at counter (local
-// slot, p / 4), gain 1 for the plain (tanh) form and 2 for the paper (ReLU)
-// form; biases and tau zero; every other slot all zero.
-__global__ void k_init_params(Dev d, Layout L) {
-  const int64_t per_slot = L.mstride / 4;
-  const int64_t total = (int64_t)d.total_slots * per_slot;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int s = (int)(i / per_slot);
-    const int q = (int)(i - (int64_t)s * per_slot);
-    const EnvDesc ed = d.env[d.env_of[s]];
-    const int ls = s - ed.slot_off;
-    float w = 0.0f;
-    if (ls < ed.init_alive && q < L.nW) {
-      const int p = layout_logical(L, q);
-      const U4 r = philox((uint32_t)ls, (uint32_t)(p >> 2), 0u, 0u, ed.seed, S_W_INIT);
-      const float fan = (float)layout_fan_in(L, q);
-      const float n = normal_of(r, p & 3);
-      w = L.relu ? n * sqrtf(__fdiv_rn(2.0f, fan)) : __fdiv_rn(n, sqrtf(fan));
-    }
-    d.master[i] = w;
-  }
-}
-
-// Streamed copy of slots [slot0, slot0 + n): BF16 elementwise (RNE), FP8 per
-// output row (scale = max|w| / 448, satfinite RNE codes), biases FP32.
-__global__ void k_requant_bf16(Dev d, Layout L, int slot0, int n) {
-  const int nW = L.nW;
-  const int per = L.nW + L.nB;
-  const int64_t total = (int64_t)n * per;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int s = slot0 + (int)(i / per);
-    const int q = (int)(i % per);
-    const float *m = d.master + (int64_t)s * (L.mstride / 4);
-    uint8_t *blk = d.wq + (int64_t)s * L.stride;
-    if (q < nW) {
-      reinterpret_cast<__nv_bfloat16 *>(blk)[q] = __float2bfloat16_rn(m[q]);
-    } else {
-      reinterpret_cast<float *>(blk + L.off_bias)[q - nW] = m[L.moff_bias / 4 + (q - nW)];
-    }
-  }
-}
-
-__global__ void k_requant_fp8(Dev d, Layout L, int slot0, int n) {
-  const int H = L.H, rows = H + L.L * H + L.A;
-  const int lane = threadIdx.x & 31;
-  // biases (and tau) are copied unchanged
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (int64_t)n * L.nB;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int s = slot0 + (int)(i / L.nB), k = (int)(i % L.nB);
-    reinterpret_cast<float *>(d.wq + (int64_t)s * L.stride + L.off_bias)[k] =
-        d.master[(int64_t)s * (L.mstride / 4) + L.moff_bias / 4 + k];
-  }
-  const int64_t warps = (int64_t)n * rows;
-  for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < warps;
-       w += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-    const int s = slot0 + (int)(w / rows);
-    const int row = (int)(w % rows);
-    const float *m = d.master + (int64_t)s * (L.mstride / 4);
-    uint8_t *blk = d.wq + (int64_t)s * L.stride;
-    int base, stride, cnt;
-    if (row < H) {  // W_in row o: elements (j, o), j < D
-      base = row; stride = H; cnt = L.D;
-    } else if (row < H + L.L * H) {  // hidden layer l, row o
-      const int l = (row - H) / H, o = (row - H) - l * H;
-      base = L.D * H + l * H * H + o; stride = H; cnt = H;
-    } else {  // head row a
-      base = L.D * H + L.L * H * H + (row - H - L.L * H) * H; stride = 1; cnt = H;
-    }
-    float mx = 0.0f;
-    for (int j = lane; j < cnt; j += 32) mx = fmaxf(mx, fabsf(m[base + j * stride]));
+    const uint32_t hi = (uint32_t)d.place_key[e];
+    const uchar4 cf = reinterpret_cast<const uchar4 *>(d.cellf)[g];
+    const uint8_t cfv[4] = {cf.x, cf.y, cf.z, cf.w};
+    const U4 r = philox((uint32_t)((c0 - ed.cell_off) >> 2), 0u, 0u, 0u, ed.seed, S_PLACE);
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, off));
-    float sc = __fdiv_rn(mx, 448.0f);
-    if (sc == 0.0f) sc = 1.0f;
-    for (int j = lane; j < cnt; j += 32) {
-      const int idx = base + j * stride;
-      blk[idx] = (uint8_t)__nv_cvt_float_to_fp8(__fdiv_rn(m[idx], sc), __NV_SATFINITE, __NV_E4M3);
+    for (int k = 0; k < 4; ++k) {
+      const uint32_t w = word_of(r, k);
+      if ((w >> 16) == hi && !(cfv[k] & CELL_WALL)) atomicAdd(&d.hist[(size_t)e * 65536 + (w & 0xFFFFu)], 1u);
     }
-    if (lane == 0) reinterpret_cast<float *>(blk + L.off_scale)[row] = sc;
   }
 }
 
-// Initial statistics: alive = K, food count, energy = K * e_init, step 0;
+// Initial statistics of environment e from the sums k_reset_world left in
+// the step's record: alive = K, food count, energy = K * e_init, step 0;
 // paper rules: energy on cells = food count * e_food; terrain rules: water
-// and biomass on cells (summed) and carried (K * w_init, K * b_body).
-__global__ void __launch_bounds__(1024) k_init_stats(Dev d, Rules R) {
-  __shared__ unsigned long long acc;
-  const int e = blockIdx.x;
+// and biomass on cells and carried (K * w_init, K * b_body).  Block-level.
+__device__ void init_stats(const Dev &d, const Rules &R, int e) {
   const EnvDesc ed = d.env[e];
-  const int n = ed.side * ed.side;
-  long long cnt = 0, water = 0, bio = 0;
-  for (int c = threadIdx.x; c < n; c += blockDim.x) {
-    cnt += (d.cellf[ed.cell_off + c] & CELL_FOOD) ? 1 : 0;
-    water += d.water[ed.cell_off + c];
-    bio += d.bio[ed.cell_off + c];
-  }
-  const long long total = block_sum_ll(cnt, &acc);
-  const long long wt = block_sum_ll(water, &acc);
-  const long long bt = block_sum_ll(bio, &acc);
   const bool terrain = R.rules == RULES_TERRAIN;
+  long long *st = d.stats_step + e * N_ST;
+  const long long total = st[ST_FOOD_TOTAL], wt = st[ST_WATER_CELLS], bt = st[ST_BIO_CELLS];
+  __syncthreads();
   for (int k = threadIdx.x; k < N_ST; k += blockDim.x) {
     long long v = 0;
     if (k == ST_ALIVE) v = ed.init_alive;
@@ -311,15 +214,173 @@ __global__ void __launch_bounds__(1024) k_init_stats(Dev d, Rules R) {
     else if (k == ST_BIO_AGENTS && terrain) v = (long long)ed.init_alive * R.b_body;
     d.stats_total[e * N_ST + k] = v;
     d.stats_last[e * N_ST + k] = v;
-    d.stats_step[e * N_ST + k] = 0;
-  }
-  if (threadIdx.x == 0) {
-    d.birth_contenders[e] = 0;
-    if (e == 0) d.counters[CNT_CONTENDERS] = 0;
-    d.place_prefix[e] = 0ull;
-    d.place_remaining[e] = ed.init_alive;
+    st[k] = 0;
   }
 }
+
+// One CTA per environment: the bin of `remaining`-th smallest digit; the
+// histogram is cleared behind the search.  Each warp reads 2,048
+// consecutive bins, 512 bytes at a time (one thread per 64 bins, whose
+// 256-byte strides left every load uncoalesced, took 69 us per digit).
+// A missing bin (fewer than K non-wall cells) sets the status word.
+// DIGIT 0: place_key = the digit, place_remaining = the rank inside the bin,
+// and the initial statistics.  DIGIT 1: place_key = the last founder's key;
+// when more cells share its draw than are needed, the CTA walks the
+// environment's cells in order to the one that fills the rank.
+template <int DIGIT>
+__global__ void __launch_bounds__(1024) k_place_find(Dev d, Rules R) {
+  __shared__ int sh[33];
+  __shared__ int found_bin, found_before, found_cnt;
+  const int e = blockIdx.x;
+  const EnvDesc ed = d.env[e];
+  if (DIGIT == 0) init_stats(d, R, e);
+  if (ed.init_alive == 0) return;
+  const int remaining = DIGIT == 0 ? ed.init_alive : d.place_remaining[e];
+  uint4 *h = reinterpret_cast<uint4 *>(d.hist + (size_t)e * 65536);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) found_bin = -1;
+  uint4 v[16];
+  int cnt = 0;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    v[i] = h[warp * 512 + i * 32 + lane];
+    cnt += (int)(v[i].x + v[i].y + v[i].z + v[i].w);
+  }
+#pragma unroll
+  for (int i = 0; i < 16; ++i) h[warp * 512 + i * 32 + lane] = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) cnt += __shfl_xor_sync(0xFFFFFFFFu, cnt, off);
+  if (lane == 0) sh[warp] = cnt;
+  __syncthreads();
+  int before = 0;
+  for (int w = 0; w < warp; ++w) before += sh[w];
+  if (before < remaining && before + cnt >= remaining) {  // this warp's bins hold it
+    int run = before;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const uint32_t w4[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+      const int own = (int)(v[i].x + v[i].y + v[i].z + v[i].w);
+      int incl = own;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const int o = __shfl_up_sync(0xFFFFFFFFu, incl, off);
+        if (lane >= off) incl += o;
+      }
+      int at = run + incl - own;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (at < remaining && at + (int)w4[k] >= remaining) {  // one lane, one bin
+          found_bin = 4 * (warp * 512 + i * 32 + lane) + k;
+          found_before = at;
+          found_cnt = (int)w4[k];
+        }
+        at += (int)w4[k];
+      }
+      run += __shfl_sync(0xFFFFFFFFu, incl, 31);
+    }
+  }
+  __syncthreads();
+  if (found_bin < 0) {
+    if (threadIdx.x == 0) {
+      atomicOr(&d.counters[CNT_STATUS], 1);
+      d.place_key[e] = DIGIT == 0 ? 0ull : ~0ull;
+      d.place_remaining[e] = remaining;
+    }
+    return;
+  }
+  const int rest = remaining - found_before;
+  if (DIGIT == 0) {
+    if (threadIdx.x == 0) {
+      d.place_key[e] = (unsigned long long)found_bin;
+      d.place_remaining[e] = rest;
+    }
+    return;
+  }
+  const uint32_t draw = (uint32_t)(d.place_key[e] << 16) | (uint32_t)found_bin;
+  __syncthreads();  // the key is read by every thread before it is replaced
+  if (rest == found_cnt) {
+    if (threadIdx.x == 0) d.place_key[e] = ((unsigned long long)draw << 32) | 0xFFFFFFFFull;
+    return;
+  }
+  const int n = ed.side * ed.side;
+  int seen = 0;
+  for (int base = 0; base < n && seen < rest; base += (int)blockDim.x) {
+    const int c = base + (int)threadIdx.x;
+    const bool hit = c < n && !(d.cellf[ed.cell_off + c] & CELL_WALL) && (uint32_t)(place_key(ed, c) >> 32) == draw;
+    int total;
+    const int at = seen + block_exclusive_scan(hit ? 1 : 0, &total, sh);
+    if (hit && at == rest - 1) d.place_key[e] = ((unsigned long long)draw << 32) | (unsigned long long)(uint32_t)c;
+    seen += total;
+  }
+}
+
+// Founders are the non-wall cells with key <= the last founder's, numbered
+// in ascending cell order.  Tiles of kPlaceTile cells, 16 consecutive cells
+// per thread; the first pass counts each tile, the second adds up the tiles
+// before it and writes, so that a large world's cells spread over the chip.
+constexpr int kPlaceTile = 4096;
+
+__device__ __forceinline__ uint32_t founder_mask(const Dev &d, const EnvDesc &ed, unsigned long long thr, int c0) {
+  uint32_t mask = 0u;
+  const int n = ed.side * ed.side;
+  for (int k = 0; k < 16 && c0 + k < n; k += 4) {
+    const uchar4 cf = *reinterpret_cast<const uchar4 *>(d.cellf + ed.cell_off + c0 + k);
+    const uint8_t cfv[4] = {cf.x, cf.y, cf.z, cf.w};
+    const U4 r = philox((uint32_t)((c0 + k) >> 2), 0u, 0u, 0u, ed.seed, S_PLACE);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const unsigned long long key =
+          ((unsigned long long)word_of(r, q) << 32) | (unsigned long long)(uint32_t)(c0 + k + q);
+      if (!(cfv[q] & CELL_WALL) && key <= thr) mask |= 1u << (k + q);
+    }
+  }
+  return mask;
+}
+
+template <bool WRITE>
+__global__ void __launch_bounds__(kPlaceTile / 16) k_place_number(Dev d) {
+  __shared__ int sh[33];
+  const int tile = blockIdx.x;
+  int lo = 0, hi = d.n_envs - 1;  // the tile's environment
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (d.env[mid].ctile_off <= tile) lo = mid;
+    else hi = mid - 1;
+  }
+  const int e = lo;
+  const EnvDesc ed = d.env[e];
+  if (ed.init_alive == 0) return;
+  const unsigned long long thr = d.place_key[e];
+  const int c0 = (tile - ed.ctile_off) * kPlaceTile + (int)threadIdx.x * 16;
+  uint32_t mask = founder_mask(d, ed, thr, c0);
+  int total;
+  if (!WRITE) {
+    block_exclusive_scan(__popc(mask), &total, sh);
+    if (threadIdx.x == 0) d.place_tiles[tile] = total;
+    return;
+  }
+  int before = 0, base;
+  for (int k = ed.ctile_off + (int)threadIdx.x; k < tile; k += blockDim.x) before += d.place_tiles[k];
+  block_exclusive_scan(before, &base, sh);
+  int at = base + block_exclusive_scan(__popc(mask), &total, sh);
+  while (mask) {
+    const int k = __ffs(mask) - 1;
+    mask &= mask - 1;
+    // the guard only matters when the select failed (status already set)
+    if (at < ed.init_alive) {
+      const int slot = ed.slot_off + at, gc = ed.cell_off + c0 + k;
+      d.pos[slot] = c0 + k;
+      d.occ[gc] = slot;
+      d.cellf[gc] |= (uint8_t)CELL_AGENT;
+    }
+    ++at;
+  }
+  const int n = ed.side * ed.side;
+  if (threadIdx.x == 0 && (tile - ed.ctile_off + 1) * kPlaceTile >= n && base + total != ed.init_alive)
+    atomicOr(&d.counters[CNT_STATUS], 2);
+}
+
+int place_tiles(int side) { return (side * side + kPlaceTile - 1) / kPlaceTile; }
 
 __global__ void k_init_static(Dev d) {
   for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < d.total_slots; s += gridDim.x * blockDim.x) {
@@ -388,42 +449,27 @@ cudaError_t launch_recount(const Dev &d, const Rules &R, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_requant(const Dev &d, const Layout &L, const Rules &R, int slot0, int n,
-                           cudaStream_t s) {
-  if (R.precision == PREC_FP32 || n <= 0) return cudaSuccess;
-  if (R.precision == PREC_BF16) {
-    const long long work = (long long)n * (L.nW + L.nB);
-    k_requant_bf16<<<grid_for(work, 256, 152 * 32), 256, 0, s>>>(d, L, slot0, n);
-  } else {
-    const long long work = (long long)n * (L.H + L.L * L.H + L.A) * 32;
-    k_requant_fp8<<<grid_for(work, 256, 152 * 32), 256, 0, s>>>(d, L, slot0, n);
-  }
-  return cudaGetLastError();
-}
-
 cudaError_t launch_reset(const Dev &d, const Layout &L, const Rules &R, const EnvGrid &g,
                          cudaStream_t s) {
   cudaError_t err;
   const int T = 256;
-  const int cb = grid_for(d.total_cells, T, g.sms * 16);
-  const int sb = grid_for(d.total_slots, T, g.sms * 16);
+  const int cb = grid_for(d.total_cells / 4 > d.total_slots ? d.total_cells / 4 : d.total_slots, T, g.sms * 8);
   if ((err = cudaMemsetAsync(d.counters, 0, sizeof(int32_t) * CNT_N, s)) != cudaSuccess) return err;
   if ((err = cudaMemsetAsync(d.step, 0, sizeof(long long), s)) != cudaSuccess) return err;
+  if ((err = cudaMemsetAsync(d.stats_step, 0, sizeof(long long) * N_ST * (size_t)d.n_envs, s)) != cudaSuccess)
+    return err;
+  if ((err = cudaMemsetAsync(d.birth_contenders, 0, sizeof(int32_t) * (size_t)d.n_envs, s)) != cudaSuccess)
+    return err;
   if ((err = cudaMemsetAsync(d.hist, 0, sizeof(uint32_t) * 65536 * (size_t)d.n_envs, s)) != cudaSuccess)
     return err;
-  k_init_cells<<<cb, T, 0, s>>>(d, R);
-  k_init_agents<<<sb, T, 0, s>>>(d, R);
-  k_init_stats<<<d.n_envs, 1024, 0, s>>>(d, R);  // also zeroes the placement prefix
-  for (int round = 0; round < 4; ++round) {
-    const int shift = 48 - 16 * round;
-    k_place_hist<<<cb, T, 0, s>>>(d, shift);
-    k_place_find<<<d.n_envs, 1024, 0, s>>>(d);
-  }
-  k_place_assign<<<d.n_envs, 1024, 0, s>>>(d);
-  const long long pw = (long long)d.total_slots * (L.mstride / 4);
-  k_init_params<<<grid_for(pw, T, g.sms * 64), T, 0, s>>>(d, L);
+  k_reset_world<<<cb, T, 0, s>>>(d, R);
+  k_place_find<0><<<d.n_envs, 1024, 0, s>>>(d, R);
+  k_place_hist<<<grid_for(d.total_cells / 4, T, g.sms * 8), T, 0, s>>>(d);
+  k_place_find<1><<<d.n_envs, 1024, 0, s>>>(d, R);
+  k_place_number<false><<<d.place_tile_count, kPlaceTile / 16, 0, s>>>(d);
+  k_place_number<true><<<d.place_tile_count, kPlaceTile / 16, 0, s>>>(d);
   if ((err = cudaGetLastError()) != cudaSuccess) return err;
-  return launch_requant(d, L, R, 0, d.total_slots, s);
+  return launch_init_params(d, L, R, s);
 }
 
 }  // namespace eco

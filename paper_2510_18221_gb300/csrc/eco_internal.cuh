@@ -162,6 +162,7 @@ struct EnvDesc {
   int32_t cell_off;   // first global cell of the environment
   int32_t init_alive;
   uint32_t seed;
+  int32_t ctile_off;  // first placement tile of the environment's cells
 };
 
 // Shape and block layout of one agent's parameters.  Logical order (the
@@ -302,8 +303,10 @@ struct Dev {
   float *master;           // [total_slots][mstride / 4]
   uint8_t *wq;             // [total_slots][stride] streamed copy (or == master)
   uint32_t *hist;          // [n_envs][65536] placement radix select
-  unsigned long long *place_prefix;  // [n_envs] (prefix, remaining)
+  unsigned long long *place_key;  // [n_envs] radix select: the first digit, then the last founder's key
   int32_t *place_remaining; // [n_envs] placement radix select
+  int32_t *place_tiles;     // [place_tile_count] founders per placement tile
+  int place_tile_count;
   uint8_t *bflag;          // [total_slots] birth pass flags
   int32_t *hp;             // [total_slots] paper rules: HP (quarter points)
   int32_t *age;            // [total_slots] paper rules: steps survived

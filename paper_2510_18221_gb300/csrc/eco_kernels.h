@@ -56,13 +56,19 @@ cudaError_t env_prepare(const Layout &L, EnvGrid *g);
 cudaError_t launch_env_phases(const Dev &d, const Layout &L, const Rules &R, const EnvGrid &g,
                               cudaStream_t s);
 
-// Reset and parameter maintenance (eco_init.cu).
+// Reset (eco_init.cu).
 cudaError_t launch_reset(const Dev &d, const Layout &L, const Rules &R, const EnvGrid &g,
                          cudaStream_t s);
 // Static per-slot tables (environment of every slot) at create.
 cudaError_t launch_init_static(const Dev &d, const EnvGrid &g, cudaStream_t s);
 // Recompute the "now" statistics (alive, food, energy, step) from the state.
 cudaError_t launch_recount(const Dev &d, const Rules &R, cudaStream_t s);
+// Placement tiles of a world of side L (reset).
+int place_tiles(int side);
+
+// Parameters (eco_params.cu): founders' weights and the streamed copy of
+// every slot; the streamed copy of slots [slot0, slot0 + n).
+cudaError_t launch_init_params(const Dev &d, const Layout &L, const Rules &R, cudaStream_t s);
 cudaError_t launch_requant(const Dev &d, const Layout &L, const Rules &R, int slot0, int n,
                            cudaStream_t s);
 
