@@ -66,10 +66,12 @@ cudaError_t launch_recount(const Dev &d, const Rules &R, cudaStream_t s);
 // Placement tiles of a world of side L (reset).
 int place_tiles(int side);
 
-// Parameters (eco_params.cu): founders' weights and the streamed copy of
-// every slot; the streamed copy of slots [slot0, slot0 + n).
+// Parameters (eco_params.cu).  Founders' weights and the streamed copy of
+// every slot; n slots from global slot slot0 out of or into `flat`, device
+// memory [n][P] in logical order (params_in also derives the streamed copy).
 cudaError_t launch_init_params(const Dev &d, const Layout &L, const Rules &R, cudaStream_t s);
-cudaError_t launch_requant(const Dev &d, const Layout &L, const Rules &R, int slot0, int n,
-                           cudaStream_t s);
+cudaError_t launch_params_in(const Dev &d, const Layout &L, const Rules &R, int slot0, int n, const float *flat,
+                             cudaStream_t s);
+cudaError_t launch_params_out(const Dev &d, const Layout &L, int slot0, int n, float *flat, cudaStream_t s);
 
 }  // namespace eco

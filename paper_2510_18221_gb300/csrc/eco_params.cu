@@ -1,7 +1,7 @@
 // eco_params.cu -- whole agents' parameters: the founders' weights (Sec.
-// 3.3: Kaiming-style initial weights, zero biases) with their streamed
-// BF16 / FP8 copy, and the re-derivation of the streamed copy from the FP32
-// masters.
+// 3.3: Kaiming-style initial weights, zero biases), the parameters a caller
+// writes (both with their streamed BF16 / FP8 copy), and the parameters a
+// caller reads.
 //
 // The logical order (the order of the Philox draws) holds a layer's weights
 // by output row, the tiled block by input, so a layer is a transposition.
@@ -35,8 +35,15 @@ __host__ __device__ inline bool tile_by4(int nin) { return (nin & 3) == 0; }
 __host__ __device__ inline int tile_stride(int nin) { return tile_by4(nin) && ((nin >> 2) & 1) == 0 ? nin + 4 : nin; }
 
 size_t tile_bytes(const Layout &L, int rows) {
-  const int a = tile_stride(L.D), b = tile_stride(L.H);
-  return 4 * ((size_t)rows * (a > b ? a : b) + 8);
+  // k_params_in's row strides and k_params_out's
+  const int nin[2] = {L.D, L.H};
+  int widest = 0;
+  for (int k = 0; k < 2; ++k) {
+    const int a = tile_stride(nin[k]), b = nin[k] | 1;
+    widest = a > widest ? a : widest;
+    widest = b > widest ? b : widest;
+  }
+  return 4 * ((size_t)rows * widest + 8);
 }
 
 // Output rows per tile: whole 32-row tiles (128-byte stores) where they fit
@@ -58,13 +65,14 @@ __device__ __forceinline__ float fp8_scale(float mx) {
 
 }  // namespace
 
-// Founders' weights: weight p = N(0,1) * sqrt(gain / fan_in) from stream
-// W_INIT at counter (local slot, p / 4), gain 1 for the plain (tanh) form and
-// 2 for the paper (ReLU) form; biases and tau zero; every other slot all
-// zero, with FP8 scales of 1.  PREC: the streamed copy derived with them
-// (BF16 elementwise RNE; FP8 per output row, scale = max|w| / 448, satfinite
-// RNE codes).
+// Parameters of slots [slot0, slot0 + n) into their blocks, with the streamed
+// copy (BF16 elementwise RNE; FP8 per output row, scale = max|w| / 448,
+// satfinite RNE codes; biases FP32).
 //
+// INIT, the founders' weights: weight p = N(0,1) * sqrt(gain / fan_in) from
+// stream W_INIT at counter (local slot, p / 4), gain 1 for the plain (tanh)
+// form and 2 for the paper (ReLU) form; biases and tau zero; every other slot
+// all zero, with FP8 scales of 1.
 // Bound by the arithmetic of the normals beside the writes: 65,536 slots of
 // 371-64-64-9 BF16 are 11.2 GB, 1.7 ms at the copy rate, and the whole reset
 // takes 4.6 ms (19.4 ms with a Philox block per element, the streamed copy
@@ -72,8 +80,12 @@ __device__ __forceinline__ float fp8_scale(float mx) {
 // founders); 683-128-128-9 FP8, 41.5 GB, 19 ms (231 ms, mostly FP8 rows read
 // with a stride).  512 threads at 64 registers: 256 or 512 threads with 2 to
 // 6 CTAs per SM lie within 5% in BF16, and up to 30% above in FP8.
-template <int PREC>
-__global__ void __launch_bounds__(kParThreads, 2) k_init_params(Dev d, Layout L, int R, int rlog) {
+//
+// Otherwise: from `flat`, [n][P] in logical order, the caller's parameters
+// on the device.
+template <int PREC, bool INIT>
+__global__ void __launch_bounds__(kParThreads, 2)
+    k_params_in(Dev d, Layout L, int R, int rlog, int slot0, int n, const float *__restrict__ flat) {
   extern __shared__ __align__(16) float tile[];
   __shared__ uint32_t s_max[kMaxRows];
   __shared__ float s_scale[kMaxRows];
@@ -88,19 +100,21 @@ __global__ void __launch_bounds__(kParThreads, 2) k_init_params(Dev d, Layout L,
   };
   const float f_vision = scale_of(0), f_internal = scale_of(L.patch * H), f_compass = scale_of((L.patch + 1) * H);
   const float f_hidden = scale_of(D * H);
-  for (int s = blockIdx.x; s < d.total_slots; s += gridDim.x) {
+  for (int i = blockIdx.x; i < n; i += gridDim.x) {
+    const int s = slot0 + i;
+    const float *in = INIT ? nullptr : flat + (int64_t)i * L.P;
     const EnvDesc ed = d.env[d.env_of[s]];
     const uint32_t ls = (uint32_t)(s - ed.slot_off);
     float *m = d.master + (int64_t)s * mper;
     uint8_t *blk = d.wq + (int64_t)s * L.stride;
-    if ((int)ls >= ed.init_alive) {  // an empty slot
+    if (INIT && (int)ls >= ed.init_alive) {  // an empty slot
       const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-      for (int i = tid; i < (int)(mper / 4); i += nt) reinterpret_cast<uint4 *>(m)[i] = z;
+      for (int k = tid; k < (int)(mper / 4); k += nt) reinterpret_cast<uint4 *>(m)[k] = z;
       if (PREC != PREC_FP32)
-        for (int i = tid; i < (int)(L.stride / 16); i += nt) reinterpret_cast<uint4 *>(blk)[i] = z;
+        for (int k = tid; k < (int)(L.stride / 16); k += nt) reinterpret_cast<uint4 *>(blk)[k] = z;
       if (PREC == PREC_FP8) {
         __syncthreads();
-        for (int i = tid; i < H + L.L * H + A; i += nt) reinterpret_cast<float *>(blk + L.off_scale)[i] = 1.0f;
+        for (int k = tid; k < H + L.L * H + A; k += nt) reinterpret_cast<float *>(blk + L.off_scale)[k] = 1.0f;
       }
       continue;
     }
@@ -111,31 +125,39 @@ __global__ void __launch_bounds__(kParThreads, 2) k_init_params(Dev d, Layout L,
       const int qbase = layer == 0 ? 0 : D * H + (layer - 1) * H * H;
       const int lrow0 = layer == 0 ? 0 : D * H + L.ns * H + (layer - 1) * (H * H + H);
       for (int o0 = 0; o0 < H; o0 += R) {
-        // 1. the rows' normals, in logical order
+        // 1. the rows (INIT: their normals), in logical order
         const int lbase = lrow0 + o0 * nin, nel = R * nin;
-        const int b0 = lbase >> 2, b1 = (lbase + nel - 1) >> 2;
-        const int shift = by4 ? 0 : lbase & 3;  // rows of a multiple of 4 start a block
-        for (int g = b0 + tid; g <= b1; g += nt) {
-          float n4[4];
-          normals4(philox(ls, (uint32_t)g, 0u, 0u, ed.seed, S_W_INIT), n4);
-          int at = 4 * (g - b0);
-          if (by4) {
-            const int rr = at / nin;
-            at += rr * (rs - nin);
+        const int shift = INIT && !by4 ? lbase & 3 : 0;  // rows of a multiple of 4 start a block
+        if (INIT) {
+          const int b0 = lbase >> 2, b1 = (lbase + nel - 1) >> 2;
+          for (int g = b0 + tid; g <= b1; g += nt) {
+            float n4[4];
+            normals4(philox(ls, (uint32_t)g, 0u, 0u, ed.seed, S_W_INIT), n4);
+            int at = 4 * (g - b0);
+            if (by4) {
+              const int rr = at / nin;
+              at += rr * (rs - nin);
+            }
+            *reinterpret_cast<float4 *>(tile + at) = make_float4(n4[0], n4[1], n4[2], n4[3]);
           }
-          *reinterpret_cast<float4 *>(tile + at) = make_float4(n4[0], n4[1], n4[2], n4[3]);
+        } else {
+          for (int rr = warp; rr < R; rr += nw)
+            for (int j = lane; j < nin; j += 32) tile[rr * rs + j] = in[lbase + rr * nin + j];
         }
         if (PREC == PREC_FP8 && tid < R) s_max[tid] = 0u;
         __syncthreads();
-        // 2. scaled, to the master (and the BF16 copy): lane = row
+        // 2. (INIT: scaled) to the master and the BF16 copy: lane = row
         const int rr = lane & (R - 1), sub = lane >> rlog, per = 32 >> rlog;
         float *row = tile + shift + rr * rs;
         float mx = 0.0f;
         auto put = [&](int j, float n) -> float {
           const int q = qbase + j * H + o0 + rr;
-          const float f = layer > 0 ? f_hidden : j < L.patch ? f_vision
-                          : (j > L.patch && j < L.patch + 5) ? f_compass : f_internal;
-          const float v = L.relu ? n * f : __fdiv_rn(n, f);
+          float v = n;
+          if (INIT) {
+            const float f = layer > 0 ? f_hidden : j < L.patch ? f_vision
+                            : (j > L.patch && j < L.patch + 5) ? f_compass : f_internal;
+            v = L.relu ? n * f : __fdiv_rn(n, f);
+          }
           m[q] = v;
           if (PREC == PREC_BF16) reinterpret_cast<__nv_bfloat16 *>(blk)[q] = __float2bfloat16_rn(v);
           if (PREC == PREC_FP8) mx = fmaxf(mx, fabsf(v));
@@ -148,12 +170,12 @@ __global__ void __launch_bounds__(kParThreads, 2) k_init_params(Dev d, Layout L,
             v.y = put(4 * c + 1, v.y);
             v.z = put(4 * c + 2, v.z);
             v.w = put(4 * c + 3, v.w);
-            if (PREC == PREC_FP8) *reinterpret_cast<float4 *>(row + 4 * c) = v;
+            if (INIT && PREC == PREC_FP8) *reinterpret_cast<float4 *>(row + 4 * c) = v;
           }
         } else {
           for (int j = warp * per + sub; j < nin; j += nw * per) {
             const float v = put(j, row[j]);
-            if (PREC == PREC_FP8) row[j] = v;
+            if (INIT && PREC == PREC_FP8) row[j] = v;
           }
         }
         if (PREC == PREC_FP8) {
@@ -185,9 +207,14 @@ __global__ void __launch_bounds__(kParThreads, 2) k_init_params(Dev d, Layout L,
     for (int a = warp; a < A; a += nw) {
       float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
       if (lane < (H >> 2)) {
-        normals4(philox(ls, (uint32_t)((out0 + a * H) >> 2) + lane, 0u, 0u, ed.seed, S_W_INIT), v);
+        if (INIT) {
+          normals4(philox(ls, (uint32_t)((out0 + a * H) >> 2) + lane, 0u, 0u, ed.seed, S_W_INIT), v);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] = L.relu ? v[k] * f_hidden : __fdiv_rn(v[k], f_hidden);
+          for (int k = 0; k < 4; ++k) v[k] = L.relu ? v[k] * f_hidden : __fdiv_rn(v[k], f_hidden);
+        } else {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) v[k] = in[out0 + a * H + 4 * lane + k];
+        }
         const int q = q3 + a * H + 4 * lane;
         *reinterpret_cast<float4 *>(m + q) = make_float4(v[0], v[1], v[2], v[3]);
         if (PREC == PREC_BF16)
@@ -208,88 +235,54 @@ __global__ void __launch_bounds__(kParThreads, 2) k_init_params(Dev d, Layout L,
         }
       }
     }
-    for (int q = L.nW + tid; q < (int)mper; q += nt) m[q] = 0.0f;
-    if (PREC != PREC_FP32)
-      for (int k = tid; k < L.nB; k += nt) reinterpret_cast<float *>(blk + L.off_bias)[k] = 0.0f;
-  }
-}
-
-// Streamed copy of slots [slot0, slot0 + n) from their masters: BF16
-// elementwise (RNE), FP8 per output row, biases FP32.
-__global__ void k_requant_bf16(Dev d, Layout L, int slot0, int n) {
-  const int nW = L.nW;
-  const int per = L.nW + L.nB;
-  const int64_t total = (int64_t)n * per;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int s = slot0 + (int)(i / per);
-    const int q = (int)(i % per);
-    const float *m = d.master + (int64_t)s * (L.mstride / 4);
-    uint8_t *blk = d.wq + (int64_t)s * L.stride;
-    if (q < nW) {
-      reinterpret_cast<__nv_bfloat16 *>(blk)[q] = __float2bfloat16_rn(m[q]);
-    } else {
-      reinterpret_cast<float *>(blk + L.off_bias)[q - nW] = m[L.moff_bias / 4 + (q - nW)];
+    // biases (and tau), and the block's padding
+    for (int k = tid; k < (int)mper - L.nW; k += nt) {
+      const float v = !INIT && k < L.nB ? in[layout_logical(L, L.nW + k)] : 0.0f;
+      m[L.nW + k] = v;
+      if (PREC != PREC_FP32 && k < L.nB) reinterpret_cast<float *>(blk + L.off_bias)[k] = v;
     }
   }
 }
 
-__global__ void k_requant_fp8(Dev d, Layout L, int slot0, int n) {
-  const int H = L.H, rows = H + L.L * H + L.A;
-  const int lane = threadIdx.x & 31;
-  // biases (and tau) are copied unchanged
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (int64_t)n * L.nB;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int s = slot0 + (int)(i / L.nB), k = (int)(i % L.nB);
-    reinterpret_cast<float *>(d.wq + (int64_t)s * L.stride + L.off_bias)[k] =
-        d.master[(int64_t)s * (L.mstride / 4) + L.moff_bias / 4 + k];
-  }
-  const int64_t warps = (int64_t)n * rows;
-  for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < warps;
-       w += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-    const int s = slot0 + (int)(w / rows);
-    const int row = (int)(w % rows);
-    const float *m = d.master + (int64_t)s * (L.mstride / 4);
-    uint8_t *blk = d.wq + (int64_t)s * L.stride;
-    int base, stride, cnt;
-    if (row < H) {  // W_in row o: elements (j, o), j < D
-      base = row; stride = H; cnt = L.D;
-    } else if (row < H + L.L * H) {  // hidden layer l, row o
-      const int l = (row - H) / H, o = (row - H) - l * H;
-      base = L.D * H + l * H * H + o; stride = H; cnt = H;
-    } else {  // head row a
-      base = L.D * H + L.L * H * H + (row - H - L.L * H) * H; stride = 1; cnt = H;
+// The masters of slots [slot0, slot0 + n) to `flat`, [n][P] in logical
+// order: the same tiles the other way, rows of an odd stride, so that 32
+// lanes writing one input of 32 rows hit 32 banks.
+__global__ void __launch_bounds__(kParThreads, 2)
+    k_params_out(Dev d, Layout L, int R, int rlog, int slot0, int n, float *__restrict__ flat) {
+  extern __shared__ __align__(16) float tile[];
+  const int D = L.D, H = L.H;
+  const int tid = threadIdx.x, nt = kParThreads, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+  const int64_t mper = L.mstride / 4;
+  for (int i = blockIdx.x; i < n; i += gridDim.x) {
+    const float *m = d.master + (int64_t)(slot0 + i) * mper;
+    float *out = flat + (int64_t)i * L.P;
+    for (int layer = 0; layer <= L.L; ++layer) {
+      const int nin = layer == 0 ? D : H, rs = nin | 1;
+      const int qbase = layer == 0 ? 0 : D * H + (layer - 1) * H * H;
+      const int lrow0 = layer == 0 ? 0 : D * H + L.ns * H + (layer - 1) * (H * H + H);
+      for (int o0 = 0; o0 < H; o0 += R) {
+        const int rr = lane & (R - 1), sub = lane >> rlog, per = 32 >> rlog;
+#pragma unroll 4
+        for (int j = warp * per + sub; j < nin; j += nw * per) tile[rr * rs + j] = m[qbase + j * H + o0 + rr];
+        __syncthreads();
+        for (int r = warp; r < R; r += nw)
+          for (int j = lane; j < nin; j += 32) out[lrow0 + (o0 + r) * nin + j] = tile[r * rs + j];
+        __syncthreads();  // the tile is reused
+      }
     }
-    float mx = 0.0f;
-    for (int j = lane; j < cnt; j += 32) mx = fmaxf(mx, fabsf(m[base + j * stride]));
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, off));
-    const float sc = fp8_scale(mx);
-    for (int j = lane; j < cnt; j += 32) {
-      const int idx = base + j * stride;
-      blk[idx] = (uint8_t)fp8_code(__fdiv_rn(m[idx], sc));
-    }
-    if (lane == 0) reinterpret_cast<float *>(blk + L.off_scale)[row] = sc;
+    // the head, the biases and tau
+    const int q3 = D * H + L.L * H * H;
+    for (int q = q3 + tid; q < L.P; q += nt) out[layout_logical(L, q)] = m[q];
   }
 }
 
-cudaError_t launch_requant(const Dev &d, const Layout &L, const Rules &R, int slot0, int n,
-                           cudaStream_t s) {
-  if (R.precision == PREC_FP32 || n <= 0) return cudaSuccess;
-  if (R.precision == PREC_BF16) {
-    const long long work = (long long)n * (L.nW + L.nB);
-    k_requant_bf16<<<grid_for(work, 256, 152 * 32), 256, 0, s>>>(d, L, slot0, n);
-  } else {
-    const long long work = (long long)n * (L.H + L.L * L.H + L.A) * 32;
-    k_requant_fp8<<<grid_for(work, 256, 152 * 32), 256, 0, s>>>(d, L, slot0, n);
-  }
-  return cudaGetLastError();
-}
-
-// Launch of one of the tiled kernels: `rows` rows of shared memory, every
-// CTA that fits.
-template <class K, class... Args>
-static cudaError_t launch_tiled(K *kernel, const Layout &L, int rows, int slots, cudaStream_t s, Args... args) {
+// Launch of one of the tiled kernels over n slots: every CTA that fits.
+template <class K, class F>
+static cudaError_t launch_tiled(K *kernel, const Dev &d, const Layout &L, int slot0, int n, F flat, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  const int rows = tile_rows(L);
+  int rlog = 3;
+  while ((1 << rlog) < rows) ++rlog;
   const size_t smem = tile_bytes(L, rows);
   cudaError_t e = cudaFuncSetAttribute((const void *)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -300,21 +293,29 @@ static cudaError_t launch_tiled(K *kernel, const Layout &L, int rows, int slots,
       cudaSuccess)
     return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  kernel<<<grid_for((long long)slots * kParThreads, kParThreads, sms * per_sm), kParThreads, smem, s>>>(args...);
+  kernel<<<n < sms * per_sm ? n : sms * per_sm, kParThreads, smem, s>>>(d, L, rows, rlog, slot0, n, flat);
   return cudaGetLastError();
 }
 
-static int log2_of(int v) {
-  int k = 0;
-  while ((1 << k) < v) ++k;
-  return k;
+template <bool INIT>
+static cudaError_t params_in(const Dev &d, const Layout &L, const Rules &R, int slot0, int n, const float *flat,
+                             cudaStream_t s) {
+  if (R.precision == PREC_FP32) return launch_tiled(k_params_in<PREC_FP32, INIT>, d, L, slot0, n, flat, s);
+  if (R.precision == PREC_BF16) return launch_tiled(k_params_in<PREC_BF16, INIT>, d, L, slot0, n, flat, s);
+  return launch_tiled(k_params_in<PREC_FP8, INIT>, d, L, slot0, n, flat, s);
 }
 
 cudaError_t launch_init_params(const Dev &d, const Layout &L, const Rules &R, cudaStream_t s) {
-  const int rows = tile_rows(L), rlog = log2_of(rows);
-  if (R.precision == PREC_FP32) return launch_tiled(k_init_params<PREC_FP32>, L, rows, d.total_slots, s, d, L, rows, rlog);
-  if (R.precision == PREC_BF16) return launch_tiled(k_init_params<PREC_BF16>, L, rows, d.total_slots, s, d, L, rows, rlog);
-  return launch_tiled(k_init_params<PREC_FP8>, L, rows, d.total_slots, s, d, L, rows, rlog);
+  return params_in<true>(d, L, R, 0, d.total_slots, nullptr, s);
+}
+
+cudaError_t launch_params_in(const Dev &d, const Layout &L, const Rules &R, int slot0, int n, const float *flat,
+                             cudaStream_t s) {
+  return params_in<false>(d, L, R, slot0, n, flat, s);
+}
+
+cudaError_t launch_params_out(const Dev &d, const Layout &L, int slot0, int n, float *flat, cudaStream_t s) {
+  return launch_tiled(k_params_out, d, L, slot0, n, flat, s);
 }
 
 }  // namespace eco
