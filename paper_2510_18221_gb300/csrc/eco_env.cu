@@ -129,15 +129,70 @@ __device__ void ph_compact_scatter(const Dev &d, int b0, int bs, int *sh, uint32
   }
 }
 
+// The scatter's first half for one tile, once the deaths are final: its alive
+// bits, this thread's place in the list and the tile's counts, without the
+// step's births.  The persistent form runs it before its last barrier, so
+// that only the children (at most kFewChildren, ascending) remain to be
+// merged behind it.
+struct TileScan {
+  uint32_t mask;  // alive bits of this thread's 16 slots
+  int at;         // alive slots before them, over all tiles
+  int base, total;  // alive slots before the tile, and in it
+};
+constexpr int kFewChildren = 32;
+
+__device__ TileScan compact_scan(const Dev &d, int tile, unsigned long long *sh /* 33 */, uint32_t t) {
+  const int32_t *cur = tile_counts_of(d, t);
+  TileScan ts;
+  ts.mask = threadIdx.x < kCompactTile / 16 ? alive_mask16(d, tile * kCompactTile + threadIdx.x * 16) : 0u;
+  int before = 0;
+  for (int k = threadIdx.x; k < tile; k += blockDim.x) before += cur[k];
+  // one scan for both: the counts before the tile in the high half
+  unsigned long long total;
+  const unsigned long long ex =
+      block_exclusive_scan64(((unsigned long long)before << 32) | (unsigned)__popc(ts.mask), &total, sh);
+  ts.base = (int)(total >> 32);
+  ts.total = (int)(uint32_t)total;
+  ts.at = ts.base + (int)(uint32_t)ex;
+  return ts;
+}
+
+__device__ void compact_write(const Dev &d, int tile, uint32_t t, TileScan ts, const int *children, int nchild) {
+  const int s0 = tile * kCompactTile + (int)threadIdx.x * 16;
+  if (threadIdx.x < kCompactTile / 16) {
+    for (int i = 0; i < nchild; ++i) {
+      const int k = children[i] - s0;
+      if (k < 0) ++ts.at;
+      else if (k < 16) ts.mask |= 1u << k;
+    }
+    while (ts.mask) {
+      const int k = __ffs(ts.mask) - 1;
+      d.alive_list[ts.at++] = s0 + k;
+      ts.mask &= ts.mask - 1;
+    }
+  }
+  if (threadIdx.x == 0) {
+    int own = 0;
+    for (int i = 0; i < nchild; ++i) own += children[i] >= s0 && children[i] < s0 + kCompactTile ? 1 : 0;
+    tile_counts_of(d, t + 1u)[tile] = ts.total + own;
+    if (tile == compact_tiles(d.total_slots) - 1) d.counters[CNT_N_ALIVE] = ts.base + ts.total + nchild;
+  }
+}
+
 // ---------------------------------------------------------------------------
 // Per-agent phases (grid-stride over the alive list).  The alive list does
-// not change until the compaction at the end of the step, so a persistent
-// thread loads the slot of its first entry once and passes it in (`first`;
-// -1 in the one-kernel-per-phase form).
+// not change until the end of the step, and between the phases only an
+// agent's own thread changes the words below, so a persistent thread keeps
+// its first agent's in registers from the move to the birth claims (each
+// phase began with a round trip to L2 for them).  The one-kernel-per-phase
+// form passes a fresh Agent, whose slot is -1, to every phase.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int agent_slot(const Dev &d, int i, int g0, int first) {
-  return (i == g0 && first >= 0) ? first : d.alive_list[i];
-}
+struct Agent {
+  int slot = -1;
+  int pos, tc, en;  // cell, move target or -1, energy
+  int act, fac;
+  bool alive;
+};
 
 // Environment of a slot (no lookup when there is one environment).
 __device__ __forceinline__ int env_index(const Dev &d, int slot) {
@@ -151,10 +206,10 @@ __device__ __forceinline__ int env_index(const Dev &d, int slot) {
 // cell, when the rules say it eats (nobody else can be on that cell); then
 // attackers claim their target cells.
 __device__ void ph_move_apply_eat(const Dev &d, const Rules &R, int n_actions, int g0, int gs, int first,
-                                  uint32_t t) {
+                                  uint32_t t, Agent &keep) {
   const int n = d.counters[CNT_N_ALIVE];
   for (int i = g0; i < n; i += gs) {
-    const int slot = agent_slot(d, i, g0, first);
+    const int slot = (i == g0 && first >= 0) ? first : d.alive_list[i];
     const int e = env_index(d, slot);
     const EnvDesc ed = d.env[e];
     const int tc = d.tgt[slot];
@@ -164,27 +219,28 @@ __device__ void ph_move_apply_eat(const Dev &d, const Rules &R, int n_actions, i
     // this thread writes them in this phase
     int en = d.energy[slot];
     const int fac = d.facing[slot];
-    // simple rules: the food bits of the cells this agent can end on, read
-    // with the claim (no other agent changes them in this phase: only the
-    // agent on a cell eats its food, and regrowth comes later)
+    // the bytes (and, paper rules, the energy) of the cells this agent can
+    // end on, read with the claim: in this phase only the agent that leaves
+    // or takes a cell, or stands on it, changes them, and regrowth comes later
     const bool eats_simple = R.rules == RULES_SIMPLE &&
                              ((R.flags & F_AUTO_EAT) || (n_actions > ACT_EAT && a == ACT_EAT));
+    const bool eats_paper = R.rules != RULES_SIMPLE && a == PA_EAT;  // an eater does not move
+    const int old = ed.cell_off + pos;
     uint32_t cf_stay = 0u, cf_move = 0u;
-    if (eats_simple) {
-      cf_stay = d.cellf[ed.cell_off + pos];
-      if (tc >= 0) cf_move = d.cellf[ed.cell_off + tc];
-    }
+    int r_stay = 0;
+    if (tc >= 0 || eats_simple || eats_paper) cf_stay = d.cellf[old];
+    if (eats_paper) r_stay = d.res[old];
     bool moved = false;
     if (tc >= 0) {
       const int gc = ed.cell_off + tc;
+      cf_move = d.cellf[gc];
       bool won = claim_local_slot(d.claim_move[gc]) == slot - ed.slot_off;
       if (R.flags & F_CANCEL_ALL) won = won && d.cnt_move[gc] == 1u;
       if (won) {
-        const int old = ed.cell_off + pos;
         d.occ[old] = -1;
-        d.cellf[old] &= (uint8_t)~CELL_AGENT;
+        d.cellf[old] = (uint8_t)(cf_stay & ~CELL_AGENT);
         d.occ[gc] = slot;
-        d.cellf[gc] |= (uint8_t)CELL_AGENT;
+        d.cellf[gc] = (uint8_t)(cf_move | CELL_AGENT);
         d.pos[slot] = tc;
         pos = tc;
         moved = true;
@@ -213,21 +269,18 @@ __device__ void ph_move_apply_eat(const Dev &d, const Rules &R, int n_actions, i
           stat_add(d.stats_step, e, ST_BIO_EATEN, bite);
         }
       }
-    } else if (R.rules != RULES_SIMPLE) {
+    } else if (eats_paper) {
       // one bite: min(e_food, energy on the cell, room in the stomach)
-      if (a == PA_EAT) {
-        const int gpos = ed.cell_off + pos;
-        const int r = d.res[gpos];
-        const int bite = min(min(R.e_food, r), R.e_cap - d.energy[slot]);
-        if (bite > 0) {
-          d.res[gpos] = r - bite;
-          d.energy[slot] += bite;
-          stat_add(d.stats_step, e, ST_EATEN, 1);
-          stat_add(d.stats_step, e, ST_EATEN_ENERGY, bite);
-          if (r == bite) {
-            d.cellf[gpos] &= (uint8_t)~CELL_FOOD;
-            stat_add(d.stats_step, e, ST_FOOD_EMPTIED, 1);
-          }
+      const int bite = min(min(R.e_food, r_stay), R.e_cap - en);
+      if (bite > 0) {
+        d.res[old] = r_stay - bite;
+        en += bite;
+        d.energy[slot] = en;
+        stat_add(d.stats_step, e, ST_EATEN, 1);
+        stat_add(d.stats_step, e, ST_EATEN_ENERGY, bite);
+        if (r_stay == bite) {
+          d.cellf[old] = (uint8_t)(cf_stay & ~CELL_FOOD);
+          stat_add(d.stats_step, e, ST_FOOD_EMPTIED, 1);
         }
       }
     } else if (eats_simple) {
@@ -269,6 +322,14 @@ __device__ void ph_move_apply_eat(const Dev &d, const Rules &R, int n_actions, i
       const U4 r = philox(t, (uint32_t)local, 0u, 0u, ed.seed, S_CLAIM_ATTACK);
       atomicMax(&d.att_cell[ed.cell_off + c], claim_key(r.x, local));
     }
+    if (i == g0) {
+      keep.slot = slot;
+      keep.pos = pos;
+      keep.tc = tc;
+      keep.en = en;
+      keep.act = a;
+      keep.fac = fac;
+    }
   }
 }
 
@@ -279,11 +340,12 @@ __device__ void ph_move_apply_eat(const Dev &d, const Rules &R, int n_actions, i
 // is, and starve_damage HP), heal only with heal_water water (spent onto the
 // cell too), and drop water and biomass at death.  One agent per cell, so
 // the cell's counters are this agent's to change here.
-__device__ __forceinline__ void health_paper(const Dev &d, const Rules &R, int slot, uint32_t t) {
-  int en = d.energy[slot];
+__device__ __forceinline__ void health_paper(const Dev &d, const Rules &R, Agent &ag, uint32_t t) {
+  const int slot = ag.slot;
+  int en = ag.en;
   int hp = d.hp[slot];
   const int age = d.age[slot];
-  const int cost = R.e_metab + (d.act[slot] != PA_REST ? R.e_act : 0);
+  const int cost = R.e_metab + (ag.act != PA_REST ? R.e_act : 0);
   int paid = cost, starved = 0, healed = 0;
   if (en >= cost) {
     en -= cost;
@@ -295,7 +357,9 @@ __device__ __forceinline__ void health_paper(const Dev &d, const Rules &R, int s
   }
   const bool terrain = R.rules == RULES_TERRAIN;
   const int e = env_index(d, slot);
-  const int gpos = d.env[e].cell_off + d.pos[slot];
+  const int gpos = d.env[e].cell_off + ag.pos;
+  // every attacker whose square covers this cell takes attack_damage
+  const int hits = (int)d.att_cell[gpos];
   int aw = terrain ? d.a_water[slot] : 0, spent = 0, thirsty = 0;
   if (terrain) {
     spent = R.w_metab;
@@ -306,8 +370,6 @@ __device__ __forceinline__ void health_paper(const Dev &d, const Rules &R, int s
     }
     aw -= spent;
   }
-  // every attacker whose square covers this cell takes attack_damage
-  const int hits = (int)d.att_cell[gpos];
   hp -= hits * R.attack_damage;
   stat_add(d.stats_step, e, ST_ATTACK_HITS, hits);
   stat_add(d.stats_step, e, ST_DAMAGE, hits * R.attack_damage);
@@ -362,6 +424,8 @@ __device__ __forceinline__ void health_paper(const Dev &d, const Rules &R, int s
   }
   d.hp[slot] = hp;
   d.energy[slot] = en;
+  ag.en = en;
+  ag.alive = hp > 0;
 }
 
 // A8 (part 2) + A9: the attack transfer, metabolism, death at e <= 0
@@ -369,19 +433,28 @@ __device__ __forceinline__ void health_paper(const Dev &d, const Rules &R, int s
 // A dying agent clears its alive flag and its cell's agent bit here, but
 // its occ entry only in the birth-claim phase, so that an attacker that
 // won the agent's cell still finds it in this phase.
-__device__ void ph_metab_death(const Dev &d, const Rules &R, int g0, int gs, int first, uint32_t t) {
+__device__ void ph_metab_death(const Dev &d, const Rules &R, int g0, int gs, uint32_t t, Agent &keep) {
   const int n = d.counters[CNT_N_ALIVE];
   for (int i = g0; i < n; i += gs) {
-    const int slot = agent_slot(d, i, g0, first);
+    Agent ag = keep;
+    if (i != g0 || keep.slot < 0) {
+      ag.slot = d.alive_list[i];
+      ag.pos = d.pos[ag.slot];
+      ag.tc = d.tgt[ag.slot];
+      ag.en = d.energy[ag.slot];
+      ag.act = d.act[ag.slot];
+      ag.fac = d.facing[ag.slot];
+    }
+    const int slot = ag.slot, tc = ag.tc;
     const int e = env_index(d, slot);
     const EnvDesc ed = d.env[e];
-    const int tc = d.tgt[slot];
     if (R.rules != RULES_SIMPLE) {
       if (tc >= 0) {
         d.claim_move[ed.cell_off + tc] = 0ull;
         if (R.flags & F_CANCEL_ALL) d.cnt_move[ed.cell_off + tc] = 0u;
       }
-      health_paper(d, R, slot, t);
+      health_paper(d, R, ag, t);
+      if (i == g0 && keep.slot >= 0) keep = ag;
       continue;
     }
     // A8 (part 2): a victim -- an agent on a claimed cell -- loses
@@ -390,15 +463,14 @@ __device__ void ph_metab_death(const Dev &d, const Rules &R, int g0, int gs, int
     // post-eat snapshot); claims are cleared in the birth-claim phase.
     // Every word this needs is final in this phase (attack claims, cells'
     // occupants and the snapshots were written before the barrier), so all
-    // are requested before the phase's first store: the slot's own words,
-    // then the claims on its own and its target cell with the target's
-    // occupant, then the occupant's snapshot.
-    int en = d.energy[slot];
-    const int pos = d.pos[slot];
-    const bool attacker = d.act[slot] == ACT_ATTACK;
-    const int fac = d.facing[slot];
+    // are requested before the phase's first store: the claims on its own
+    // and its target cell with the target's occupant, then the occupant's
+    // snapshot.
+    int en = ag.en;
+    const int pos = ag.pos;
+    const bool attacker = ag.act == ACT_ATTACK;
     const unsigned long long hit = d.att_cell[ed.cell_off + pos];
-    const int c = ed.cell_off + step_cell(pos, fac, ed.side);
+    const int c = attacker ? ed.cell_off + step_cell(pos, ag.fac, ed.side) : ed.cell_off + pos;
     const bool won = attacker && claim_local_slot(d.att_cell[c]) == slot - ed.slot_off;
     const int v = attacker ? d.occ[c] : -1;
     if (tc >= 0) {
@@ -413,16 +485,22 @@ __device__ void ph_metab_death(const Dev &d, const Rules &R, int g0, int gs, int
       stat_add(d.stats_step, e, ST_ENERGY_TRANSFERRED, g);
     }
     en = en - loss + g - R.e_metab;
-    if (en <= 0) {
+    const bool alive = en > 0;
+    if (!alive) {
       const int gpos = ed.cell_off + pos;
       d.alive[slot] = 0;
       atomicSub(&tile_counts_of(d, t)[slot / kCompactTile], 1);
-      d.cellf[gpos] &= (uint8_t)~CELL_AGENT;
+      // an atomic on the cell's word: regrowth sets food bits in this phase
+      atomicAnd(reinterpret_cast<unsigned *>(d.cellf) + (gpos >> 2), ~(CELL_AGENT << (8 * (gpos & 3))));
       stat_add(d.stats_step, e, ST_DEATHS, 1);
       stat_add(d.stats_step, e, ST_DEAD_ENERGY, en);
       en = 0;
     }
     d.energy[slot] = en;
+    if (i == g0 && keep.slot >= 0) {
+      keep.en = en;
+      keep.alive = alive;
+    }
   }
 }
 
@@ -430,41 +508,44 @@ __device__ void ph_metab_death(const Dev &d, const Rules &R, int g0, int gs, int
 // reproduce; terrain rules: that also carry b_body + b_child biomass and
 // w_child water) claim the free non-wall cell behind them and join their
 // environment's contender list.
-__device__ void ph_birth_claim(const Dev &d, const Rules &R, int g0, int gs, int first, uint32_t t) {
+__device__ void ph_birth_claim(const Dev &d, const Rules &R, int g0, int gs, uint32_t t, const Agent &keep) {
   const int n = d.counters[CNT_N_ALIVE];
   for (int i = g0; i < n; i += gs) {
-    const int slot = agent_slot(d, i, g0, first);
-    {
-      // clear this step's attack claims and, for an agent that died, its
-      // cell's occupant (kept for the attackers of the metabolism phase)
-      const EnvDesc ed = d.env[env_index(d, slot)];
-      const int pos = d.pos[slot];
-      const int a = d.act[slot];
-      if (!d.alive[slot]) d.occ[ed.cell_off + pos] = -1;
-      if (R.rules != RULES_SIMPLE) {
-        if (a == PA_ATTACK) {
-          const int side = ed.side;
-          const int px = pos % side, py = pos / side;
-          const int f = d.facing[slot], rt = (f + 1) & 3;
-          for (int fw = 1; fw <= 3; ++fw)
-            for (int lat = -1; lat <= 1; ++lat) {
-              const int cx = wrapi(px + fw * dir_dx(f) + lat * dir_dx(rt), side);
-              const int cy = wrapi(py + fw * dir_dy(f) + lat * dir_dy(rt), side);
-              d.att_cell[ed.cell_off + cy * side + cx] = 0ull;
-            }
-        }
-      } else if (a == ACT_ATTACK) {
-        d.att_cell[ed.cell_off + step_cell(pos, d.facing[slot], ed.side)] = 0ull;
+    Agent ag = keep;
+    if (i != g0 || keep.slot < 0) {
+      ag.slot = d.alive_list[i];
+      ag.pos = d.pos[ag.slot];
+      ag.en = d.energy[ag.slot];
+      ag.act = d.act[ag.slot];
+      ag.fac = d.facing[ag.slot];
+      ag.alive = d.alive[ag.slot] != 0;
+    }
+    const int slot = ag.slot, pos = ag.pos;
+    const int e = env_index(d, slot);
+    const EnvDesc ed = d.env[e];
+    // clear this step's attack claims and, for an agent that died, its
+    // cell's occupant (kept for the attackers of the metabolism phase)
+    if (!ag.alive) d.occ[ed.cell_off + pos] = -1;
+    if (R.rules != RULES_SIMPLE) {
+      if (ag.act == PA_ATTACK) {
+        const int side = ed.side;
+        const int px = pos % side, py = pos / side;
+        const int f = ag.fac, rt = (f + 1) & 3;
+        for (int fw = 1; fw <= 3; ++fw)
+          for (int lat = -1; lat <= 1; ++lat) {
+            const int cx = wrapi(px + fw * dir_dx(f) + lat * dir_dx(rt), side);
+            const int cy = wrapi(py + fw * dir_dy(f) + lat * dir_dy(rt), side);
+            d.att_cell[ed.cell_off + cy * side + cx] = 0ull;
+          }
       }
+    } else if (ag.act == ACT_ATTACK) {
+      d.att_cell[ed.cell_off + step_cell(pos, ag.fac, ed.side)] = 0ull;
     }
     int bt = -1;
-    if (d.alive[slot] && d.energy[slot] >= R.e_repro &&
-        (R.rules == RULES_SIMPLE || d.act[slot] == PA_REPRODUCE) &&
+    if (ag.alive && ag.en >= R.e_repro && (R.rules == RULES_SIMPLE || ag.act == PA_REPRODUCE) &&
         (R.rules != RULES_TERRAIN ||
          (d.a_bio[slot] >= R.b_body + R.b_child && d.a_water[slot] >= R.w_child))) {
-      const int e = env_index(d, slot);
-      const EnvDesc ed = d.env[e];
-      const int c = step_cell(d.pos[slot], (d.facing[slot] + 2) & 3, ed.side);
+      const int c = step_cell(pos, (ag.fac + 2) & 3, ed.side);
       const int gc = ed.cell_off + c;
       if (!(d.cellf[gc] & (CELL_WALL | CELL_AGENT))) {
         const int local = slot - ed.slot_off;
@@ -498,6 +579,7 @@ constexpr int kMaxFastTiles = 256;
 
 struct BirthSmem {
   int sh[33];
+  unsigned long long sh64[33];
   int win[kBirthCap];
   int free_[kBirthCap];
   int nwin, nborn, nfree;
@@ -892,8 +974,35 @@ size_t mutate_smem_bytes(const Layout &L) {
 }
 
 // A12: regrowth of food on non-wall food-less cells; four cells per thread
-// share one Philox block (counter (step, local cell / 4)).
-__device__ void ph_regrow(const Dev &d, const Rules &R, int g0, int gs, uint32_t t) {
+// share one Philox block (counter (step, local cell / 4)).  Under the simple
+// rules nothing but eating changes a food bit, so it may run beside the
+// deaths: both change their bits of a cell's word by atomics.
+__device__ __forceinline__ uint32_t regrow_draw(const EnvDesc &ed, int c0, uint32_t thr, uint32_t t) {
+  const U4 r = philox(t, (uint32_t)((c0 - ed.cell_off) >> 2), 0u, 0u, ed.seed, S_REGROW);
+  return (r.x < thr ? 1u : 0u) | (r.y < thr ? 2u : 0u) | (r.z < thr ? 4u : 0u) | (r.w < thr ? 8u : 0u);
+}
+
+// The draws of this thread's first kRegrowAhead groups, four bits each: they
+// depend on the step alone, and a million cells' Philox blocks are 2 us of
+// the whole chip's arithmetic, so the persistent form draws them while the
+// agents' threads wait for memory.
+constexpr int kRegrowAhead = 8;
+
+__device__ uint32_t regrow_draws(const Dev &d, const Rules &R, int g0, int gs, uint32_t t) {
+  uint32_t draws = 0u;
+  if (R.thr_regrow == 0u) return draws;
+#pragma unroll 1
+  for (int k = 0; k < kRegrowAhead; ++k) {
+    const int g = g0 + k * gs;
+    if (g >= (d.total_cells >> 2)) break;
+    const EnvDesc ed = d.env[d.n_envs == 1 ? 0 : env_of_cell(d.env, d.n_envs, g << 2)];
+    draws |= regrow_draw(ed, g << 2, R.thr_regrow, t) << (4 * k);
+  }
+  return draws;
+}
+
+// `ahead` groups of this thread have their draws in `draws`.
+__device__ void ph_regrow(const Dev &d, const Rules &R, int g0, int gs, uint32_t t, uint32_t draws, int ahead) {
   const int groups = d.total_cells >> 2;
   if (R.rules != RULES_TERRAIN) {
     // kRG of this thread's groups per round, their cell bytes loaded
@@ -901,9 +1010,9 @@ __device__ void ph_regrow(const Dev &d, const Rules &R, int g0, int gs, uint32_t
     // previous group's); the regrown count is kept per environment and
     // added once per environment (groups ascend, so environments do).
     constexpr int kRG = 4;
-    int e = -1, grown_e = 0;
+    int e = -1, grown_e = 0, done = 0;
     EnvDesc ed = d.env[0];
-    for (int gb = g0; gb < groups; gb += kRG * gs) {
+    for (int gb = g0; gb < groups; gb += kRG * gs, done += kRG) {
       uchar4 cfv[kRG];
 #pragma unroll
       for (int k = 0; k < kRG; ++k) {
@@ -922,21 +1031,20 @@ __device__ void ph_regrow(const Dev &d, const Rules &R, int g0, int gs, uint32_t
           ed = d.env[e];
         }
         uchar4 cf = cfv[k];
-        const bool any = !((cf.x & (CELL_WALL | CELL_FOOD)) && (cf.y & (CELL_WALL | CELL_FOOD)) &&
-                           (cf.z & (CELL_WALL | CELL_FOOD)) && (cf.w & (CELL_WALL | CELL_FOOD)));
-        if (!any) continue;
-        const U4 r = philox(t, (uint32_t)((c0 - ed.cell_off) >> 2), 0u, 0u, ed.seed, S_REGROW);
-        int mask = 0;
-        if (!(cf.x & (CELL_WALL | CELL_FOOD)) && r.x < R.thr_regrow) { cf.x |= CELL_FOOD; mask |= 1; }
-        if (!(cf.y & (CELL_WALL | CELL_FOOD)) && r.y < R.thr_regrow) { cf.y |= CELL_FOOD; mask |= 2; }
-        if (!(cf.z & (CELL_WALL | CELL_FOOD)) && r.z < R.thr_regrow) { cf.z |= CELL_FOOD; mask |= 4; }
-        if (!(cf.w & (CELL_WALL | CELL_FOOD)) && r.w < R.thr_regrow) { cf.w |= CELL_FOOD; mask |= 8; }
+        constexpr uint32_t kNo = CELL_WALL | CELL_FOOD;
+        uint32_t mask = (cf.x & kNo ? 0u : 1u) | (cf.y & kNo ? 0u : 2u) | (cf.z & kNo ? 0u : 4u) | (cf.w & kNo ? 0u : 8u);
+        if (!mask) continue;
+        mask &= done + k < ahead ? (draws >> (4 * (done + k))) & 15u : regrow_draw(ed, c0, R.thr_regrow, t);
         if (!mask) continue;
         grown_e += __popc(mask);
-        if (R.rules == RULES_PAPER)  // one bite of energy on each regrown cell
+        if (R.rules == RULES_PAPER) {  // one bite of energy on each regrown cell
           for (int q = 0; q < 4; ++q)
-            if (mask & (1 << q)) d.res[c0 + q] = R.e_food;
-        reinterpret_cast<uchar4 *>(d.cellf)[g] = cf;
+            if (mask & (1u << q)) d.res[c0 + q] = R.e_food;
+        }
+        unsigned bits = 0u;
+        for (int q = 0; q < 4; ++q)
+          if (mask & (1u << q)) bits |= CELL_FOOD << (8 * q);
+        atomicOr(reinterpret_cast<unsigned *>(d.cellf) + g, bits);
       }
     }
     if (e >= 0) stat_add(d.stats_step, e, ST_REGROWN, grown_e);
@@ -962,7 +1070,8 @@ __device__ void ph_regrow(const Dev &d, const Rules &R, int g0, int gs, uint32_t
       e = env_of_cell(d.env, d.n_envs, c0);
       ed = d.env[e];
     }
-    uchar4 cf = reinterpret_cast<uchar4 *>(d.cellf)[g];
+    const uchar4 cf4 = reinterpret_cast<const uchar4 *>(d.cellf)[g];
+    uint8_t cf[4] = {cf4.x, cf4.y, cf4.z, cf4.w};
     // the group's biomass, remainders and energy, loaded together (the
     // loads are independent; the chain per cell was the phase's cost)
     int bio[4], res[4];
@@ -976,28 +1085,25 @@ __device__ void ph_regrow(const Dev &d, const Rules &R, int g0, int gs, uint32_t
       pho[0] = p4.x, pho[1] = p4.y, pho[2] = p4.z, pho[3] = p4.w;
     }
     int grown = 0;
-    const bool any = !((cf.x & (CELL_WALL | CELL_FOOD)) && (cf.y & (CELL_WALL | CELL_FOOD)) &&
-                       (cf.z & (CELL_WALL | CELL_FOOD)) && (cf.w & (CELL_WALL | CELL_FOOD)));
     // a zero threshold (no random regrowth) grows nothing: no draw needed
-    if (any && R.thr_regrow != 0u) {
-      const U4 r = philox(t, (uint32_t)((c0 - ed.cell_off) >> 2), 0u, 0u, ed.seed, S_REGROW);
-      int mask = 0;
-      if (!(cf.x & (CELL_WALL | CELL_FOOD)) && r.x < R.thr_regrow) { cf.x |= CELL_FOOD; mask |= 1; }
-      if (!(cf.y & (CELL_WALL | CELL_FOOD)) && r.y < R.thr_regrow) { cf.y |= CELL_FOOD; mask |= 2; }
-      if (!(cf.z & (CELL_WALL | CELL_FOOD)) && r.z < R.thr_regrow) { cf.z |= CELL_FOOD; mask |= 4; }
-      if (!(cf.w & (CELL_WALL | CELL_FOOD)) && r.w < R.thr_regrow) { cf.w |= CELL_FOOD; mask |= 8; }
-      grown = __popc(mask);
+    if (R.thr_regrow != 0u) {
+      const uint32_t mask = regrow_draw(ed, c0, R.thr_regrow, t);
+#pragma unroll
       for (int k = 0; k < 4; ++k)  // one bite of energy on each regrown cell, in the group's registers
-        if (mask & (1 << k)) res[k] = R.e_food;
+        if ((mask & (1u << k)) && !(cf[k] & (CELL_WALL | CELL_FOOD))) {
+          cf[k] |= (uint8_t)CELL_FOOD;
+          res[k] = R.e_food;
+          ++grown;
+        }
     }
     bool changed = grown != 0;
     // energy grows on free biomass: a 2^-16 fixed-point remainder per cell
     // makes the sum over steps exact; at most res_cap energy per cell
-    uint8_t *cfb = reinterpret_cast<uint8_t *>(&cf);
     bool touched = grown != 0;
+#pragma unroll
     for (int k = 0; k < 4; ++k) {
       const int b = bio[k];
-      if ((cfb[k] & CELL_WALL) || b <= 0) continue;
+      if ((cf[k] & CELL_WALL) || b <= 0) continue;
       const unsigned long long acc = (unsigned long long)pho[k] + (unsigned long long)b * (unsigned)R.photo_q16;
       pho[k] = (uint32_t)(acc & 0xFFFFull);
       touched = true;
@@ -1005,7 +1111,7 @@ __device__ void ph_regrow(const Dev &d, const Rules &R, int g0, int gs, uint32_t
       const long long gain = min((long long)(acc >> 16), (long long)R.res_cap - r);
       if (gain <= 0) continue;
       if (r == 0) {
-        cfb[k] |= (uint8_t)CELL_FOOD;
+        cf[k] |= (uint8_t)CELL_FOOD;
         ++refilled_e;
         changed = true;
       }
@@ -1016,7 +1122,7 @@ __device__ void ph_regrow(const Dev &d, const Rules &R, int g0, int gs, uint32_t
       reinterpret_cast<int4 *>(d.res)[g] = make_int4(res[0], res[1], res[2], res[3]);
       reinterpret_cast<uint4 *>(d.photo)[g] = make_uint4(pho[0], pho[1], pho[2], pho[3]);
     }
-    if (changed) reinterpret_cast<uchar4 *>(d.cellf)[g] = cf;
+    if (changed) reinterpret_cast<uchar4 *>(d.cellf)[g] = make_uchar4(cf[0], cf[1], cf[2], cf[3]);
     grown_e += grown;
   }
   flush();
@@ -1034,21 +1140,20 @@ __device__ void ph_regrow(const Dev &d, const Rules &R, int g0, int gs, uint32_t
 // four): the group, the four cells above and below it (16-byte loads) and
 // the two at its ends are loaded together, so a group costs one round
 // trip of independent loads.  Other sides take the neighbours one by one.
-__device__ __forceinline__ uint32_t flow_pick(int w, long long here, const long long hn[4], const bool wn[4]) {
-  long long lowest = 0;
-  int best = -1;
+// Surfaces are below 2^31 + 2^16 (water counts are int32, rock heights below
+// 2^16), so 32-bit unsigned arithmetic holds them exactly.
+__device__ __forceinline__ uint32_t flow_pick(int w, uint32_t here, const uint32_t hn[4], const bool wn[4]) {
+  uint32_t lowest = 0xFFFFFFFFu;
+  uint32_t best = 0u;
 #pragma unroll
   for (int dir = 0; dir < 4; ++dir) {
-    if (wn[dir]) continue;
-    if (best < 0 || hn[dir] < lowest) {
-      best = dir;
-      lowest = hn[dir];
+    const uint32_t h = wn[dir] ? 0xFFFFFFFFu : hn[dir];
+    if (h < lowest) {
+      best = (uint32_t)dir;
+      lowest = h;
     }
   }
-  if (best >= 0 && lowest < here) {
-    const long long amount = min((here - lowest) / 5, (long long)w);
-    return ((uint32_t)amount << 2) | (uint32_t)best;
-  }
+  if (lowest < here) return (min((here - lowest) / 5u, (uint32_t)w) << 2) | best;
   return 0u;
 }
 
@@ -1078,59 +1183,52 @@ __device__ void ph_flow_out(const Dev &d, int g0, int gs) {
   const int groups = d.total_cells >> 2;
   for (int g = g0; g < groups; g += gs) {
     const int c0 = g << 2;
-    int w[4];
+    const EnvDesc ed = d.env[env_of_cell(d.env, d.n_envs, c0)];
+    int w[4], rk[4];
     unpack4(reinterpret_cast<const int4 *>(d.water)[g], w);
+    unpack4(reinterpret_cast<const int4 *>(d.rock)[g], rk);
     const uchar4 cf4 = reinterpret_cast<const uchar4 *>(d.cellf)[g];
     const uint8_t cf[4] = {cf4.x, cf4.y, cf4.z, cf4.w};
-    bool wet[4], any = false;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      wet[k] = w[k] > 0 && !(cf[k] & CELL_WALL);
-      any |= wet[k];
-    }
     uint32_t f[4] = {0u, 0u, 0u, 0u};
-    if (any) {
-      const EnvDesc ed = d.env[env_of_cell(d.env, d.n_envs, c0)];
-      int rk[4];
-      unpack4(reinterpret_cast<const int4 *>(d.rock)[g], rk);
-      if ((ed.side & 3) == 0) {
-        const FlowGroup fg = flow_group(ed, c0);
-        int wu[4], ru[4], wd[4], rd[4];
-        unpack4(*reinterpret_cast<const int4 *>(d.water + fg.up0), wu);
-        unpack4(*reinterpret_cast<const int4 *>(d.rock + fg.up0), ru);
-        unpack4(*reinterpret_cast<const int4 *>(d.water + fg.dn0), wd);
-        unpack4(*reinterpret_cast<const int4 *>(d.rock + fg.dn0), rd);
-        const uchar4 cu = *reinterpret_cast<const uchar4 *>(d.cellf + fg.up0);
-        const uchar4 cd = *reinterpret_cast<const uchar4 *>(d.cellf + fg.dn0);
-        const uint8_t cuv[4] = {cu.x, cu.y, cu.z, cu.w}, cdv[4] = {cd.x, cd.y, cd.z, cd.w};
-        const long long hw = (long long)d.rock[fg.west] + d.water[fg.west];
-        const long long he = (long long)d.rock[fg.east] + d.water[fg.east];
-        const bool ww = (d.cellf[fg.west] & CELL_WALL) != 0, we = (d.cellf[fg.east] & CELL_WALL) != 0;
+    if ((ed.side & 3) == 0) {
+      // every load at once: waiting for the group's own water first, to
+      // skip dry groups, put a second round trip into every wet one
+      const FlowGroup fg = flow_group(ed, c0);
+      int wu[4], ru[4], wd[4], rd[4];
+      unpack4(*reinterpret_cast<const int4 *>(d.water + fg.up0), wu);
+      unpack4(*reinterpret_cast<const int4 *>(d.rock + fg.up0), ru);
+      unpack4(*reinterpret_cast<const int4 *>(d.water + fg.dn0), wd);
+      unpack4(*reinterpret_cast<const int4 *>(d.rock + fg.dn0), rd);
+      const uchar4 cu = *reinterpret_cast<const uchar4 *>(d.cellf + fg.up0);
+      const uchar4 cd = *reinterpret_cast<const uchar4 *>(d.cellf + fg.dn0);
+      const uint8_t cuv[4] = {cu.x, cu.y, cu.z, cu.w}, cdv[4] = {cd.x, cd.y, cd.z, cd.w};
+      const uint32_t hw = (uint32_t)d.rock[fg.west] + (uint32_t)d.water[fg.west];
+      const uint32_t he = (uint32_t)d.rock[fg.east] + (uint32_t)d.water[fg.east];
+      const bool ww = (d.cellf[fg.west] & CELL_WALL) != 0, we = (d.cellf[fg.east] & CELL_WALL) != 0;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          if (!wet[k]) continue;
-          // N, E, S, W
-          const long long hn[4] = {(long long)ru[k] + wu[k],
-                                   k < 3 ? (long long)rk[k + 1] + w[k + 1] : he,
-                                   (long long)rd[k] + wd[k],
-                                   k > 0 ? (long long)rk[k - 1] + w[k - 1] : hw};
-          const bool wn[4] = {(cuv[k] & CELL_WALL) != 0, k < 3 ? (cf[k + 1] & CELL_WALL) != 0 : we,
-                              (cdv[k] & CELL_WALL) != 0, k > 0 ? (cf[k - 1] & CELL_WALL) != 0 : ww};
-          f[k] = flow_pick(w[k], (long long)rk[k] + w[k], hn, wn);
+      for (int k = 0; k < 4; ++k) {
+        if (w[k] <= 0 || (cf[k] & CELL_WALL)) continue;
+        // N, E, S, W
+        const uint32_t hn[4] = {(uint32_t)ru[k] + (uint32_t)wu[k],
+                                k < 3 ? (uint32_t)rk[k + 1] + (uint32_t)w[k + 1] : he,
+                                (uint32_t)rd[k] + (uint32_t)wd[k],
+                                k > 0 ? (uint32_t)rk[k - 1] + (uint32_t)w[k - 1] : hw};
+        const bool wn[4] = {(cuv[k] & CELL_WALL) != 0, k < 3 ? (cf[k + 1] & CELL_WALL) != 0 : we,
+                            (cdv[k] & CELL_WALL) != 0, k > 0 ? (cf[k - 1] & CELL_WALL) != 0 : ww};
+        f[k] = flow_pick(w[k], (uint32_t)rk[k] + (uint32_t)w[k], hn, wn);
+      }
+    } else {
+      for (int k = 0; k < 4; ++k) {
+        if (w[k] <= 0 || (cf[k] & CELL_WALL)) continue;
+        const int lc = c0 + k - ed.cell_off;
+        uint32_t hn[4];
+        bool wn[4];
+        for (int dir = 0; dir < 4; ++dir) {
+          const int n = ed.cell_off + step_cell(lc, dir, ed.side);
+          wn[dir] = (d.cellf[n] & CELL_WALL) != 0;
+          hn[dir] = (uint32_t)d.rock[n] + (uint32_t)d.water[n];
         }
-      } else {
-        for (int k = 0; k < 4; ++k) {
-          if (!wet[k]) continue;
-          const int lc = c0 + k - ed.cell_off;
-          long long hn[4];
-          bool wn[4];
-          for (int dir = 0; dir < 4; ++dir) {
-            const int n = ed.cell_off + step_cell(lc, dir, ed.side);
-            wn[dir] = (d.cellf[n] & CELL_WALL) != 0;
-            hn[dir] = (long long)d.rock[n] + d.water[n];
-          }
-          f[k] = flow_pick(w[k], (long long)rk[k] + w[k], hn, wn);
-        }
+        f[k] = flow_pick(w[k], (uint32_t)rk[k] + (uint32_t)w[k], hn, wn);
       }
     }
     reinterpret_cast<uint4 *>(d.flow)[g] = make_uint4(f[0], f[1], f[2], f[3]);
@@ -1150,7 +1248,6 @@ __device__ void ph_flow_in(const Dev &d, int g0, int gs) {
     const int c0 = g << 2;
     const uchar4 cf4 = reinterpret_cast<const uchar4 *>(d.cellf)[g];
     const uint8_t cf[4] = {cf4.x, cf4.y, cf4.z, cf4.w};
-    if ((cf[0] & cf[1] & cf[2] & cf[3]) & CELL_WALL) continue;
     int w[4];
     unpack4(reinterpret_cast<const int4 *>(d.water)[g], w);
     const uint4 f4 = reinterpret_cast<const uint4 *>(d.flow)[g];
@@ -1202,64 +1299,73 @@ __device__ void reset_birth_counters(const Dev &d) {
   }
 }
 
-// A13: fold this step's counters into the per-environment records and
-// advance the step counter (one CTA).  Agent-steps and attacks come from the
-// action histogram the policy kernel counted.
-// reset_counters: also clear this step's birth counters (the one-kernel-
-// per-phase form; the persistent form clears them at its next launch's
-// start, because its other CTAs may still read them here).
-__device__ void ph_finish(const Dev &d, const Rules &R, bool reset_counters) {
-  const long long t = d.step[0];
-  for (int i = threadIdx.x; i < d.n_envs; i += blockDim.x) {
-    long long *st = d.stats_step + i * N_ST;
-    long long as = 0;
-    for (int a = 0; a < 16; ++a) as += st[ST_ACT0 + a];
-    st[ST_AGENT_STEPS] = as;
-    st[ST_ATTACKS] = st[ST_ACT0 + (R.rules != RULES_SIMPLE ? PA_ATTACK : ACT_ATTACK)];
+// A13: fold this step's counters into environment e's records, one warp:
+// lane l holds the statistics l and l + 32, read together, and the derived
+// ones are exchanged by shuffles, so the fold costs one round trip and no
+// block barrier.  born, failed: births the step's record does not hold yet
+// (the fast birth path).  Agent-steps and attacks come from the action
+// histogram the policy kernel counted.
+__device__ void fold_env(const Dev &d, const Rules &R, int e, long long t, int born, int failed) {
+  static_assert(N_ST <= 64, "two statistics per lane");
+  const int lane = threadIdx.x & 31;
+  const bool paper = R.rules != RULES_SIMPLE;
+  long long *st = d.stats_step + e * N_ST;
+  long long *tot = d.stats_total + e * N_ST;
+  long long *last = d.stats_last + e * N_ST;
+  long long s[2], o[2];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int k = lane + 32 * q;
+    s[q] = k < N_ST ? st[k] : 0;
+    o[q] = k < N_ST ? tot[k] : 0;
+    if (k == ST_BIRTHS) s[q] += born;
+    if (k == ST_FAILED_BIRTHS) s[q] += failed;
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < d.n_envs * N_ST; i += blockDim.x) {
-    const int e = i / N_ST, k = i - e * N_ST;
-    long long *st = d.stats_step + e * N_ST;
-    long long *tot = d.stats_total + e * N_ST;
-    long long *last = d.stats_last + e * N_ST;
-    long long v;
+  auto step_of = [&](int k) { return __shfl_sync(0xFFFFFFFFu, k < 32 ? s[0] : s[1], k & 31); };
+  static_assert(ST_ACT0 + 16 <= 32, "the action counts lie in the first half");
+  long long as = lane >= ST_ACT0 && lane < ST_ACT0 + 16 ? s[0] : 0;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) as += __shfl_xor_sync(0xFFFFFFFFu, as, off);
+  const long long attacks = step_of(ST_ACT0 + (paper ? PA_ATTACK : ACT_ATTACK));
+  const long long births = step_of(ST_BIRTHS), deaths = step_of(ST_DEATHS), dead_e = step_of(ST_DEAD_ENERGY);
+  const long long eaten = step_of(ST_EATEN), grown = step_of(ST_REGROWN);
+  const long long emptied = step_of(ST_FOOD_EMPTIED), refilled = step_of(ST_FOOD_REFILLED);
+  const long long eaten_e = step_of(ST_EATEN_ENERGY), paid = step_of(ST_METAB_PAID), heals = step_of(ST_HEALS);
+  const long long photo = step_of(ST_PHOTO);
+  // the flow moves water between cells only
+  const long long water = step_of(ST_WATER_SPENT) + step_of(ST_DEAD_WATER) - step_of(ST_DRUNK);
+  const long long bio = step_of(ST_DEAD_BIO) - step_of(ST_BIO_EATEN);
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int k = lane + 32 * q;
+    if (k >= N_ST) break;
+    long long v = o[q], l;
     if (k == ST_STEP) {
       v = t + 1;
     } else if (k == ST_ALIVE) {
-      v = tot[k] + st[ST_BIRTHS] - st[ST_DEATHS];
+      v += births - deaths;
     } else if (k == ST_FOOD_TOTAL) {
-      v = R.rules != RULES_SIMPLE ? tot[k] + st[ST_REGROWN] - st[ST_FOOD_EMPTIED] + st[ST_FOOD_REFILLED]
-                                 : tot[k] + st[ST_REGROWN] - st[ST_EATEN];
+      v += paper ? grown - emptied + refilled : grown - eaten;
     } else if (k == ST_ENERGY_TOTAL) {
-      v = R.rules != RULES_SIMPLE
-              ? tot[k] + st[ST_EATEN_ENERGY] - st[ST_METAB_PAID] - (long long)R.heal_cost * st[ST_HEALS] -
-                    st[ST_DEAD_ENERGY]
-              : tot[k] + (long long)R.e_food * st[ST_EATEN] - (long long)R.e_metab * st[ST_AGENT_STEPS] -
-                    st[ST_DEAD_ENERGY];
+      v += paper ? eaten_e - paid - (long long)R.heal_cost * heals - dead_e
+                 : (long long)R.e_food * eaten - (long long)R.e_metab * as - dead_e;
     } else if (k == ST_RES_TOTAL) {
-      v = R.rules != RULES_SIMPLE ? tot[k] + (long long)R.e_food * st[ST_REGROWN] - st[ST_EATEN_ENERGY] +
-                                        st[ST_DEAD_ENERGY] + st[ST_PHOTO]
-                                  : 0;
+      v = paper ? v + (long long)R.e_food * grown - eaten_e + dead_e + photo : 0;
     } else if (k == ST_WATER_CELLS || k == ST_WATER_AGENTS) {
-      // the flow moves water between cells only
-      const long long to_cells = st[ST_WATER_SPENT] + st[ST_DEAD_WATER] - st[ST_DRUNK];
-      v = tot[k] + (k == ST_WATER_CELLS ? to_cells : -to_cells);
+      v += k == ST_WATER_CELLS ? water : -water;
     } else if (k == ST_BIO_CELLS || k == ST_BIO_AGENTS) {
-      const long long to_cells = st[ST_DEAD_BIO] - st[ST_BIO_EATEN];
-      v = tot[k] + (k == ST_BIO_CELLS ? to_cells : -to_cells);
+      v += k == ST_BIO_CELLS ? bio : -bio;
     } else {
-      last[k] = st[k];
-      tot[k] += st[k];
+      l = k == ST_AGENT_STEPS ? as : k == ST_ATTACKS ? attacks : s[q];
+      last[k] = l;
+      tot[k] = v + l;
+      st[k] = 0;
       continue;
     }
     last[k] = v;
     tot[k] = v;
+    st[k] = 0;
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < d.n_envs * N_ST; i += blockDim.x) d.stats_step[i] = 0;
-  if (threadIdx.x == 0) d.step[0] = t + 1;
-  if (reset_counters) reset_birth_counters(d);
 }
 
 // ---------------------------------------------------------------------------
@@ -1276,9 +1382,18 @@ __global__ void __launch_bounds__(256) k_compact_scatter(Dev d) {
   ph_compact_scatter(d, blockIdx.x, gridDim.x, sh, (uint32_t)d.step[0], nullptr, 0, nullptr);
 }
 #define STEP_T ((uint32_t)d.step[0])
-__global__ void k_move_apply_eat(Dev d, Rules R, int A) { ph_move_apply_eat(d, R, A, GRID_ARGS, -1, STEP_T); }
-__global__ void k_metab_death(Dev d, Rules R) { ph_metab_death(d, R, GRID_ARGS, -1, STEP_T); }
-__global__ void k_birth_claim(Dev d, Rules R) { ph_birth_claim(d, R, GRID_ARGS, -1, STEP_T); }
+__global__ void k_move_apply_eat(Dev d, Rules R, int A) {
+  Agent none;
+  ph_move_apply_eat(d, R, A, GRID_ARGS, -1, STEP_T, none);
+}
+__global__ void k_metab_death(Dev d, Rules R) {
+  Agent none;
+  ph_metab_death(d, R, GRID_ARGS, STEP_T, none);
+}
+__global__ void k_birth_claim(Dev d, Rules R) {
+  Agent none;
+  ph_birth_claim(d, R, GRID_ARGS, STEP_T, none);
+}
 __global__ void __launch_bounds__(1024) k_birth_assign(Dev d, Rules R) {
   __shared__ BirthSmem S;
   ph_birth_assign(d, R, blockIdx.x, gridDim.x, S, STEP_T);
@@ -1288,10 +1403,15 @@ __global__ void __launch_bounds__(256) k_mutate(Dev d, Layout L, Rules R) {
   __shared__ float s_scale[kMutRows];
   ph_mutate(d, L, R, blockIdx.x, gridDim.x, msm, s_scale, STEP_T, nullptr, nullptr, 0);
 }
-__global__ void k_regrow(Dev d, Rules R) { ph_regrow(d, R, GRID_ARGS, STEP_T); }
+__global__ void k_regrow(Dev d, Rules R) { ph_regrow(d, R, GRID_ARGS, STEP_T, 0u, 0); }
 __global__ void k_flow_out(Dev d) { ph_flow_out(d, GRID_ARGS); }
 __global__ void k_flow_in(Dev d) { ph_flow_in(d, GRID_ARGS); }
-__global__ void k_finish(Dev d, Rules R) { ph_finish(d, R, true); }
+__global__ void __launch_bounds__(1024) k_finish(Dev d, Rules R) {
+  const long long t = d.step[0];
+  for (int e = threadIdx.x >> 5; e < d.n_envs; e += blockDim.x >> 5) fold_env(d, R, e, t, 0, 0);
+  reset_birth_counters(d);  // synchronises the CTA: every thread has read the step
+  if (threadIdx.x == 0) d.step[0] = t + 1;
+}
 #undef STEP_T
 
 // ---------------------------------------------------------------------------
@@ -1319,7 +1439,6 @@ __device__ bool grid_sync(unsigned *count, int *status_word, unsigned nblocks, u
   if (threadIdx.x == 0) {
     cuda::atomic_ref<unsigned, cuda::thread_scope_device> cnt(*count);
     const unsigned target = k * nblocks;
-    __threadfence();
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
     unsigned it = 0, v;
     int ok = 1;
@@ -1405,6 +1524,75 @@ __device__ void fast_births(const Dev &d, BirthSmem &S, int nc) {
   __syncthreads();
 }
 
+// fast_births for at most 32 claimants, by the CTA's first warp: a lane per
+// claimant, ranks by comparison, no block barrier but the last (the sort's
+// and the scan's were most of the path's time).
+__device__ void fast_births_few(const Dev &d, BirthSmem &S, int nc) {
+  if (threadIdx.x < 32) {
+    const EnvDesc ed = d.env[0];
+    const int lane = threadIdx.x;
+    const int g = lane < nc ? d.contenders[ed.slot_off + lane] : 0x7FFFFFFF;
+    const int bt = lane < nc ? d.bcell[ed.slot_off + lane] : 0;
+    // free slots before each tile: eight tiles per lane
+    constexpr int kPer = kMaxFastTiles / 32;
+    const int tiles = (ed.n_slots + kCompactTile - 1) / kCompactTile;
+    int f[kPer], own = 0;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      f[k] = lane * kPer + k < tiles ? d.free_tiles[lane * kPer + k] : 0;
+      own += f[k];
+    }
+    const bool won = lane < nc && claim_local_slot(d.claim_birth[ed.cell_off + bt]) == g - ed.slot_off;
+    int incl = own;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int o = __shfl_up_sync(0xFFFFFFFFu, incl, off);
+      if (lane >= off) incl += o;
+    }
+    const int nfree = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    int before = incl - own;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      S.tile_first[lane * kPer + k] = before;
+      before += f[k];
+    }
+    int rank = 0;
+#pragma unroll
+    for (int l = 0; l < 32; ++l) {
+      const int o = __shfl_sync(0xFFFFFFFFu, won ? g : 0x7FFFFFFF, l);
+      rank += o < g ? 1 : 0;
+    }
+    const int nwin = __popc(__ballot_sync(0xFFFFFFFFu, won));
+    if (won) S.win[rank] = g;
+    __syncwarp();
+    const int nborn = nwin < nfree ? nwin : nfree;
+    if (lane < nborn) {
+      int k = 0;
+      while (k + 1 < tiles && S.tile_first[k + 1] <= lane) ++k;
+      S.free_[lane] = ed.slot_off + d.free_list[k * kFastBirths + (lane - S.tile_first[k])];
+    }
+    if (lane == 0) {
+      S.nwin = nwin;
+      S.nfree = nfree;
+      S.nborn = nborn;
+    }
+  }
+  __syncthreads();
+}
+
+// Request a plane into L2: 2 KB pieces, consecutive ones by different CTAs
+// (c of n; one SM alone asks for 50 GB/s).
+__device__ __forceinline__ void prefetch_cells(const void *plane, long long bytes, int c, int n) {
+  constexpr long long kPiece = 2048;
+  for (long long at = ((long long)threadIdx.x * n + c) * kPiece; at < (bytes & ~15ll);
+       at += (long long)blockDim.x * n * kPiece) {
+    const long long left = (bytes & ~15ll) - at;
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(reinterpret_cast<const uint8_t *>(plane) + at),
+                 "r"((uint32_t)(left < kPiece ? left : kPiece))
+                 : "memory");
+  }
+}
+
 __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long v;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(v));
@@ -1467,7 +1655,12 @@ __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rul
   };
   // Housekeeping goes to CTAs with little else to do in its interval: the
   // per-agent phases take one agent per thread from CTA 0 on, and the
-  // alive list's tiles go to CTAs 0 .. tiles - 1.
+  // alive list's tiles go to CTAs 0 .. tiles - 1.  The cells' phases leave
+  // the CTAs with agents out where those are at most half.
+  const int agent_ctas = (n_alive + (int)blockDim.x - 1) / (int)blockDim.x;
+  const int cell_first = agent_ctas * 2 <= (int)nb ? agent_ctas : 0;
+  const int cg0 = g0 - cell_first * (int)blockDim.x, cgs = gs - cell_first * (int)blockDim.x;
+  const bool cell_cta = (int)blockIdx.x >= cell_first;
   const int tiles = compact_tiles(d.total_slots);
   const unsigned last = nb - 1u;
   const unsigned fold_cta = (unsigned)tiles < nb ? (unsigned)tiles : 0u;      // statistics
@@ -1480,17 +1673,39 @@ __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rul
     if (threadIdx.x == 0) d.barrier[BAR_COUNT0 + ((t + 1u) & 1u)] = 0u;
   }
   const int first = g0 < n_alive ? first_entry : -1;
-  ph_move_apply_eat(d, R, L.A, g0, gs, first, t);
+  Agent ag;
+  uint32_t draws = 0u;
+  ph_move_apply_eat(d, R, L.A, g0, gs, first, t, ag);
+  if (cell_cta) {
+    if (R.rules != RULES_TERRAIN) {
+      draws = regrow_draws(d, R, cg0, cgs, t);
+    } else {
+      // the policy kernel's weight stream has pushed the cells' planes out of
+      // L2: bring them back ahead of the cells' phases
+      const int cc = (int)blockIdx.x - cell_first, ncc = (int)nb - cell_first;
+      prefetch_cells(d.cellf, d.total_cells, cc, ncc);
+      prefetch_cells(d.bio, 4 * (long long)d.total_cells, cc, ncc);
+      prefetch_cells(d.res, 4 * (long long)d.total_cells, cc, ncc);
+      prefetch_cells(d.photo, 4 * (long long)d.total_cells, cc, ncc);
+      prefetch_cells(d.water, 4 * (long long)d.total_cells, cc, ncc);
+      prefetch_cells(d.rock, 4 * (long long)d.total_cells, cc, ncc);
+    }
+  }
   if (!sync()) return;
-  ph_metab_death(d, R, g0, gs, first, t);
+  ph_metab_death(d, R, g0, gs, t, ag);
+  // simple rules: only eating takes food, and it is over
+  if (R.rules == RULES_SIMPLE && cell_cta) ph_regrow(d, R, cg0, cgs, t, draws, kRegrowAhead);
   if (!sync()) return;
-  // regrowth (with photosynthesis and the flow's transfers) needs only the
-  // state after the deaths, and birth claims read only wall and agent bits,
-  // which regrowth keeps: the two share an interval
-  ph_birth_claim(d, R, g0, gs, first, t);
+  // regrowth under the other rules (with photosynthesis and the flow's
+  // transfers) needs the state after the deaths, and birth claims read only
+  // wall and agent bits, which regrowth keeps: the two share an interval,
+  // and with them what the births need to know of the slots
+  ph_birth_claim(d, R, g0, gs, t, ag);
   if (d.n_envs == 1 && compact_tiles(d.total_slots) <= kMaxFastTiles) list_free_slots(d, S.sh);
-  ph_regrow(d, R, g0, gs, t);
-  if (R.rules == RULES_TERRAIN) ph_flow_out(d, g0, gs);
+  TileScan ts = {0u, 0, 0, 0};
+  if (tiles <= (int)nb && (int)blockIdx.x < tiles) ts = compact_scan(d, blockIdx.x, S.sh64, t);
+  if (R.rules != RULES_SIMPLE && cell_cta) ph_regrow(d, R, cg0, cgs, t, draws, kRegrowAhead);
+  if (R.rules == RULES_TERRAIN && cell_cta) ph_flow_out(d, cg0, cgs);
   if (!sync()) return;
   // Every claim is in, and the count of claimants does not change again
   // in this launch, so every CTA takes the same branch.
@@ -1504,17 +1719,17 @@ __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rul
     ph_birth_assign(d, R, blockIdx.x, gridDim.x, S, t);
     if (!sync()) return;
   } else if (fast) {
-    fast_births(d, S, claimants);
+    if (claimants <= 32) fast_births_few(d, S, claimants);
+    else fast_births(d, S, claimants);
   }
-  // Every statistic of the step is in (the fast path's births are counted
-  // here): one CTA folds them while the others go on.
+  // Every statistic of the step is in: one CTA folds them, a warp per
+  // environment from its last warp on, while the others go on.
   if (blockIdx.x == fold_cta) {
-    if (fast && threadIdx.x == 0) {
-      d.stats_step[ST_BIRTHS] += S.nborn;
-      d.stats_step[ST_FAILED_BIRTHS] += S.nwin - S.nborn;
+    const int nw = (int)blockDim.x >> 5;
+    for (int e = nw - 1 - ((int)threadIdx.x >> 5); e < d.n_envs; e += nw) {
+      fold_env(d, R, e, (long long)t, fast ? S.nborn : 0, fast ? S.nwin - S.nborn : 0);
+      if (e == 0 && (threadIdx.x & 31) == 0) d.step[0] = (long long)t + 1;
     }
-    __syncthreads();
-    ph_finish(d, R, false);
   }
   if (fast) {
     // the births' side effects, pair by pair over every thread of the grid
@@ -1532,7 +1747,12 @@ __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rul
   // launch, so no barrier follows.  Mutation work starts from the last CTA,
   // the alive list from the first.
   if (R.rules == RULES_TERRAIN) ph_flow_in(d, g0, gs);
-  ph_compact_scatter(d, blockIdx.x, gridDim.x, S.sh, t, fast ? S.free_ : nullptr, fast ? S.nborn : 0, S.cmask);
+  const int nchild = fast ? S.nborn : 0;
+  if (tiles <= (int)nb && (claimants == 0 || (fast && nchild <= kFewChildren))) {
+    if ((int)blockIdx.x < tiles) compact_write(d, blockIdx.x, t, ts, S.free_, nchild);
+  } else {
+    ph_compact_scatter(d, blockIdx.x, gridDim.x, S.sh, t, fast ? S.free_ : nullptr, nchild, S.cmask);
+  }
   if (claimants > 0) {
     if (R.precision != PREC_FP8)
       ph_mutate_flat(d, L, R, t, fast ? S.win : nullptr, fast ? S.free_ : nullptr, fast ? S.nborn : 0,

@@ -521,6 +521,37 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int *total, int *sh /
   return excl;
 }
 
+// The same of one 64-bit value per thread.
+__device__ __forceinline__ unsigned long long block_exclusive_scan64(unsigned long long v, unsigned long long *total,
+                                                                     unsigned long long *sh /* >= 33 */) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nwarps = blockDim.x >> 5;
+  unsigned long long incl = v;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const unsigned long long o = __shfl_up_sync(0xFFFFFFFFu, incl, off);
+    if (lane >= off) incl += o;
+  }
+  if (lane == 31) sh[warp] = incl;
+  __syncthreads();
+  if (warp == 0) {
+    const unsigned long long w = lane < nwarps ? sh[lane] : 0ull;
+    unsigned long long wi = w;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const unsigned long long o = __shfl_up_sync(0xFFFFFFFFu, wi, off);
+      if (lane >= off) wi += o;
+    }
+    if (lane < nwarps) sh[lane] = wi - w;
+    if (lane == 31) sh[32] = wi;
+  }
+  __syncthreads();
+  const unsigned long long excl = sh[warp] + incl - v;
+  *total = sh[32];
+  __syncthreads();
+  return excl;
+}
+
 // Launch helpers (host).
 int grid_for(long long n, int threads, int max_blocks);
 
