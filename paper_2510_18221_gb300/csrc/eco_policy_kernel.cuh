@@ -191,12 +191,9 @@ struct Log2<1> {
 // holds H / 32 finished outputs, so the bias, scale and activation run on
 // all 32 lanes.
 template <int PREC, int H>
-__device__ __forceinline__ void layer_finish(float *acc, const float *__restrict__ bias, int nbias,
-                                             const float *__restrict__ scale, float *__restrict__ out,
-                                             int lane, int relu) {
+__device__ __forceinline__ void finish_sums(float *acc, int lane) {
   constexpr int E = Unit<PREC>::E;
   constexpr int UPJ = H / E;
-  int base = 0;
 #pragma unroll
   for (int step = 0; (UPJ << step) < 32; ++step) {
     const int off = UPJ << step;
@@ -209,10 +206,28 @@ __device__ __forceinline__ void layer_finish(float *acc, const float *__restrict
       const float keep = upper ? hi : lo;
       acc[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, upper ? lo : hi, off);
     }
-    if (upper) base += half;
   }
+}
+
+// The first of the H / 32 outputs that finish_sums leaves this lane.
+template <int PREC, int H>
+__device__ __forceinline__ int finish_first(int lane) {
+  constexpr int E = Unit<PREC>::E;
+  constexpr int UPJ = H / E;
+  int o = (lane & (UPJ - 1)) * E;
+#pragma unroll
+  for (int step = 0; (UPJ << step) < 32; ++step)
+    if (lane & (UPJ << step)) o += E >> (step + 1);
+  return o;
+}
+
+template <int PREC, int H>
+__device__ __forceinline__ void layer_finish(float *acc, const float *__restrict__ bias, int nbias,
+                                             const float *__restrict__ scale, float *__restrict__ out,
+                                             int lane, int relu) {
+  finish_sums<PREC, H>(acc, lane);
   constexpr int NOUT = H / 32;
-  const int o0 = (lane & (UPJ - 1)) * E + base;
+  const int o0 = finish_first<PREC, H>(lane);
 #pragma unroll
   for (int i = 0; i < NOUT; ++i) {
     const int o = o0 + i;
@@ -326,6 +341,50 @@ __device__ __forceinline__ int nbr_cell(int px, int py, int dir, int L) {
   return y * L + x;
 }
 
+// Where the cells of one agent's patch lie: cell c (row-major, the row far
+// ahead first) is fw cells ahead of the agent and ri to its right.  Away from
+// the seams -- nearly every agent of a large world -- the cell index is linear
+// in fw and ri, two multiply-adds in place of two wrapped coordinates and
+// their product (the gather was a tenth of an FP8 agent's instructions).
+struct Patch {
+  int px, py, side, pos;
+  int ax, ay, bx, by;  // one cell ahead, one to the right
+  int A, B;            // the same as index steps
+  int fw0, RR, k;
+  uint32_t kdiv;       // ceil(2^32 / k): c / k by a multiply-high, exact for c < 2^10
+  bool inside;         // no cell of the patch lies across a seam
+
+  __device__ __forceinline__ Patch(const Rules &R, int side_, int pos_, int f, uint32_t kdiv_) {
+    side = side_;
+    pos = pos_;
+    k = R.patch_k;
+    kdiv = kdiv_;
+    RR = k >> 1;
+    py = pos / side;
+    px = pos - py * side;
+    // an unrotated patch is the one of an agent facing north
+    const int g = (R.flags & F_ROTATE_OBS) ? f : 0, rt = (g + 1) & 3;
+    ax = dir_dx(g), ay = dir_dy(g), bx = dir_dx(rt), by = dir_dy(rt);
+    A = ay * side + ax;
+    B = by * side + bx;
+    // rows run from far ahead (top) to behind (Around) or to the agent's
+    // own row (Front); columns from the agent's left to its right
+    fw0 = R.view == VIEW_FRONT ? k - 1 : RR;
+    inside = px >= fw0 && px < side - fw0 && py >= fw0 && py < side - fw0;
+  }
+  // Env-local index of the patch's cell c.
+  __device__ __forceinline__ int cell(int c) const {
+    const int r = (int)__umulhi((uint32_t)c, kdiv), col = c - r * k;
+    const int fw = fw0 - r, ri = col - RR;
+    if (inside) return pos + fw * A + ri * B;
+    // |offsets| <= k - 1 < side: one correction wraps the torus
+    int cx = px + fw * ax + ri * bx, cy = py + fw * ay + ri * by;
+    cx += cx < 0 ? side : (cx >= side ? -side : 0);
+    cy += cy < 0 ? side : (cy >= side ? -side : 0);
+    return cy * side + cx;
+  }
+};
+
 // Observation of one agent (Sec. 3.2 "Sensors"): the k x k x nch patch
 // (row, column, channel), then the scalars, into xs.  Lanes 0..3 also read
 // the flags of the four neighbouring cells (N E S W) for the move claim:
@@ -333,41 +392,21 @@ __device__ __forceinline__ int nbr_cell(int px, int py, int dir, int L) {
 __device__ __forceinline__ void gather_obs(const Dev &d, const Layout &L, const Rules &R, int slot,
                                            int env, int pos, int f, float *xs, int lane,
                                            uint32_t kdiv, int *nb_cell, uint32_t *nb_flags) {
-  const int k = R.patch_k, RR = k >> 1, kk = k * k;
-  const bool rotate = (R.flags & F_ROTATE_OBS) != 0;
+  const int kk = R.patch_k * R.patch_k;
   const EnvDesc ed = d.env[env];
-  const int side = ed.side;
-  const int px = pos % side, py = pos / side;
-  const int rt = (f + 1) & 3;
+  const Patch pt(R, ed.side, pos, f, kdiv);
   const uint8_t *cellf = d.cellf + ed.cell_off;
   if (lane < 4) {
-    *nb_cell = nbr_cell(px, py, lane, side);
+    *nb_cell = nbr_cell(pt.px, pt.py, lane, ed.side);
     *nb_flags = cellf[*nb_cell];
   }
-  // rows run from far ahead (top) to behind (Around) or to the agent's
-  // own row (Front); columns from the agent's left to its right
-  const int fw0 = R.view == VIEW_FRONT ? k - 1 : RR;
   const int nch = L.nch;
   const bool terrain = R.rules == RULES_TERRAIN;
   const int rock0 = terrain ? d.rock[ed.cell_off + pos] : 0;
   for (int c = lane; c < kk; c += 32) {
-    // c / k by a multiply-high with ceil(2^32 / k): exact for c < 2^10
-    const int r = (int)__umulhi((uint32_t)c, kdiv), col = c - r * k;
-    int dx, dy;
-    if (rotate) {
-      const int fw = fw0 - r, ri = col - RR;
-      dx = fw * dir_dx(f) + ri * dir_dx(rt);
-      dy = fw * dir_dy(f) + ri * dir_dy(rt);
-    } else {
-      dx = col - RR;
-      dy = r - RR;
-    }
-    // |dx|, |dy| <= k / 2 < side: one correction wraps the torus
-    int cx = px + dx, cy = py + dy;
-    cx += cx < 0 ? side : (cx >= side ? -side : 0);
-    cy += cy < 0 ? side : (cy >= side ? -side : 0);
-    const int gc = ed.cell_off + cy * side + cx;
-    const uint32_t cf = cellf[cy * side + cx];
+    const int lc = pt.cell(c);
+    const int gc = ed.cell_off + lc;
+    const uint32_t cf = cellf[lc];
     if (R.vision == VISION_RGB) {
       // rendered colours: the occupant's colour trait, else grey wall,
       // else green food (terrain: the cell's biomass, energy and water)
@@ -431,6 +470,106 @@ __device__ __forceinline__ void gather_obs(const Dev &d, const Layout &L, const 
     }
     xs[nch * kk + lane] = v;
   }
+}
+
+// The one-hot observation of gather_obs under the simple rules in two halves,
+// so that its loads can be in flight while another agent is computed: a
+// lane's cells lane, lane + 32, ... of a patch of at most 32 * kCellsAhead,
+// the neighbours' flags and the energy.
+constexpr int kCellsAhead = 4;  // 11 x 11 patches and below
+struct CellsAhead {
+  uint32_t cell[kCellsAhead];
+  int nb_cell, energy;
+  uint32_t nb_flags;
+};
+
+__device__ __forceinline__ void cells_load(const Dev &d, const Rules &R, int slot, int env, int pos, int f, int lane,
+                                           uint32_t kdiv, CellsAhead &ca) {
+  const int kk = R.patch_k * R.patch_k;
+  const EnvDesc ed = d.env[d.n_envs == 1 ? 0 : env];
+  const Patch pt(R, ed.side, pos, f, kdiv);
+  const uint8_t *cellf = d.cellf + ed.cell_off;
+  ca.nb_cell = 0;
+  ca.nb_flags = 0u;
+  if (lane < 4) {
+    ca.nb_cell = nbr_cell(pt.px, pt.py, lane, ed.side);
+    ca.nb_flags = cellf[ca.nb_cell];
+  }
+#pragma unroll
+  for (int q = 0; q < kCellsAhead; ++q) {
+    const int c = lane + 32 * q;
+    ca.cell[q] = c < kk ? cellf[pt.cell(c)] : 0u;
+  }
+  ca.energy = lane == 0 ? d.energy[slot] : 0;
+}
+
+__device__ __forceinline__ void cells_store(const Rules &R, const Layout &L, const CellsAhead &ca, int f, float *xs,
+                                            int lane) {
+  const int kk = R.patch_k * R.patch_k;
+#pragma unroll
+  for (int q = 0; q < kCellsAhead; ++q) {
+    const int c = lane + 32 * q;
+    if (c < kk) {
+      xs[3 * c + 0] = (ca.cell[q] & CELL_FOOD) ? 1.0f : 0.0f;
+      xs[3 * c + 1] = (ca.cell[q] & CELL_AGENT) ? 1.0f : 0.0f;
+      xs[3 * c + 2] = (ca.cell[q] & CELL_WALL) ? 1.0f : 0.0f;
+    }
+  }
+  if (lane < R.n_scalars) {
+    float v = 0.0f;
+    if (lane == 0) v = (float)ca.energy / (float)R.e_repro;
+    else if (R.n_scalars >= 8 && lane == 1 + f) v = 1.0f;
+    xs[3 * kk + lane] = v;
+  }
+}
+
+// The same for the input-sparse kernels: the list of the nonzero inputs in
+// ascending order, straight from the cells' bits (a warp ballot per channel
+// and 32 cells, instead of writing every input to shared memory and balloting
+// over 32 at a time), and the values of the listed inputs alone in xs.
+// Returns their number.  48,000 agents, BF16, variant 8: 134 -> 119 us.
+__device__ __forceinline__ int cells_list(const Rules &R, const CellsAhead &ca, int f, float *xs, short *idx, int lane) {
+  const int kk = R.patch_k * R.patch_k;
+  const unsigned below = (1u << lane) - 1u;
+  int n = 0;
+#pragma unroll
+  for (int q = 0; q < kCellsAhead; ++q) {
+    const uint32_t cf = ca.cell[q];  // 0 past the patch
+    const unsigned food = __ballot_sync(0xFFFFFFFFu, (cf & CELL_FOOD) != 0u);
+    const unsigned agent = __ballot_sync(0xFFFFFFFFu, (cf & CELL_AGENT) != 0u);
+    const unsigned wall = __ballot_sync(0xFFFFFFFFu, (cf & CELL_WALL) != 0u);
+    if (cf & (CELL_FOOD | CELL_AGENT | CELL_WALL)) {
+      int at = n + __popc(food & below) + __popc(agent & below) + __popc(wall & below);
+      const int j = 3 * (lane + 32 * q);
+      if (cf & CELL_FOOD) idx[at++] = (short)j, xs[j] = 1.0f;
+      if (cf & CELL_AGENT) idx[at++] = (short)(j + 1), xs[j + 1] = 1.0f;
+      if (cf & CELL_WALL) idx[at++] = (short)(j + 2), xs[j + 2] = 1.0f;
+    }
+    n += __popc(food) + __popc(agent) + __popc(wall);
+  }
+  float v = 0.0f;
+  if (lane == 0) v = (float)ca.energy / (float)R.e_repro;
+  else if (R.n_scalars >= 8 && lane == 1 + f) v = 1.0f;
+  const unsigned nz = __ballot_sync(0xFFFFFFFFu, v != 0.0f);
+  if (v != 0.0f) {
+    idx[n + __popc(nz & below)] = (short)(3 * kk + lane);
+    xs[3 * kk + lane] = v;
+  }
+  return n + __popc(nz);
+}
+
+// The list of the nonzero inputs of an observation in xs, in ascending order
+// (a warp ballot per 32).
+__device__ __forceinline__ int list_nonzero(int D, const float *xs, short *idx, int lane) {
+  int n = 0;
+  for (int base = 0; base < D; base += 32) {
+    const int j = base + lane;
+    const bool nz = j < D && xs[j] != 0.0f;
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, nz);
+    if (nz) idx[n + __popc(m & ((1u << lane) - 1u))] = (short)j;
+    n += __popc(m);
+  }
+  return n;
 }
 
 // One group of 32 head units (output-major rows of UPJ units): unit u of
@@ -599,6 +738,8 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
   // agent starts with its observation gather.  (A slot's facing is written
   // only by the warp that computes it, in its own iteration.)
   int i = w0 < G_eff ? w0 : n_alive;
+  // one-hot vision under the simple rules: cells_list's short cut
+  const bool ahead = R.vision == VISION_CHANNELS && R.rules == RULES_SIMPLE && k * k <= 32 * kCellsAhead;
   int slot_n = 0, env_n = 0, pos_n = 0, f_n = 0;
   if (i < n_alive) {
     slot_n = d.alive_list[i];
@@ -616,7 +757,21 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
     }
     int nb_cell = 0;
     uint32_t nb_flags = 0;
-    gather_obs(d, L, R, slot, env, pos, f, xs, lane, kdiv, &nb_cell, &nb_flags);
+    [[maybe_unused]] short *idx = reinterpret_cast<short *>(ls + 16);
+    [[maybe_unused]] int n_nz = 0;
+    if (SPARSE && ahead) {
+      CellsAhead ca;
+      cells_load(d, R, slot, env, pos, f, lane, kdiv, ca);
+      n_nz = cells_list(R, ca, f, xs, idx, lane);
+      nb_cell = ca.nb_cell;
+      nb_flags = ca.nb_flags;
+    } else {
+      gather_obs(d, L, R, slot, env, pos, f, xs, lane, kdiv, &nb_cell, &nb_flags);
+      if constexpr (SPARSE) {
+        __syncwarp();
+        n_nz = list_nonzero(L.D, xs, idx, lane);
+      }
+    }
     __syncwarp();
 
     const uint8_t *blk = d.wq + (int64_t)slot * L.stride;
@@ -626,17 +781,6 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
 
     // -- input layer: act(sum over sensors of (W_s x_s + b_s)) -> hs
     if constexpr (SPARSE) {
-      // list the nonzero inputs in ascending order (a warp ballot per 32)
-      short *idx = reinterpret_cast<short *>(ls + 16);
-      int n_nz = 0;
-      for (int base = 0; base < L.D; base += 32) {
-        const int j = base + lane;
-        const bool nz = j < L.D && xs[j] != 0.0f;
-        const unsigned m = __ballot_sync(0xFFFFFFFFu, nz);
-        if (nz) idx[n_nz + __popc(m & ((1u << lane) - 1u))] = (short)j;
-        n_nz += __popc(m);
-      }
-      __syncwarp();
       layer_in_major<PREC, H, UNROLL, true>(wb + L.off_w1 / 16, n_nz, xs, bias, L.ns, scale, hs,
                                             lane, L.relu, idx);
     } else {
@@ -694,22 +838,291 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
 }
 
 // ---------------------------------------------------------------------------
+// The ring form: each lane copies its own units into a ring in shared memory
+// (cp.async, 16 bytes per lane and row of 32 units), NB batches of UB rows
+// ahead of the products, across layers and into the warp's next agent.  The
+// copies in flight need no registers and never drain between batches, so
+// the stream goes on while the warp samples, gathers and starts its next
+// agent, and an agent's first weights are on their way before its
+// observation is.  A lane reads only what it copied itself: no barrier.
+// Lanes take the same units in the same order as in k_policy, so logits,
+// actions and state are bit-identical to it.
+//
+// us per launch on GB300, register form (the autotuner's pick) -> ring:
+// 371-64-64-9 FP8 300 agents 13 -> 11, 2,000 19 -> 15, 12,000 66 -> 63, 48,000
+// 220 -> 212; BF16 300 17 -> 11, 2,000 27 -> 25, 48,000 382 -> 397;
+// 683-128-128-9 FP8 300 41 -> 19, 2,000 49 -> 43.  Between 3,040 and 4,864
+// agents the register form holds them all at once and the ring takes two
+// rounds (FP8, 4,500: 27 -> 33).  (A ring per warp filled by bulk copies with
+// mbarriers lost above 2,500 agents: 150 ns per chunk and warp for the wait,
+// the warp barrier and the next copy.)
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ uint4 lds_unit(uint32_t addr) {
+  uint4 r;
+  asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
+               : "r"(addr)
+               : "memory");
+  return r;
+}
+
+// Batches of an agent: every section (W_in, each hidden layer, the head)
+// starts a batch, and its last batch may be short.
+__host__ __device__ inline int ring_batches(int units, int ub) { return (units + 32 * ub - 1) / (32 * ub); }
+
+template <int PREC, int H, int NB, int UB, bool SPARSE>
+struct Ring {
+  static constexpr uint32_t kBytes = NB * UB * 512u;
+  static constexpr int UPJ = H / Unit<PREC>::E;
+  uint32_t lane0, pos;        // shared address of this lane's unit in row 0; ring offset of the batch at hand
+  int sec, left;              // being copied: section (0 W_in, 1..L hidden, L + 1 head), batches left of it
+  uint32_t off, lim;          // this lane's next byte in the block, and the section's end
+  const uint8_t *src, *nxt;   // the block being copied, and the one after it (null: none)
+
+  // (SPARSE: W_in's rows depend on the observation and are loaded directly.)
+  __device__ __forceinline__ void start(const Layout &L, int lane) {
+    sec = SPARSE ? 1 : 0;
+    left = ring_batches((SPARSE ? H : L.D) * UPJ, UB);
+    off = (SPARSE ? (uint32_t)L.off_w2 : 0u) + 16u * (uint32_t)lane;
+    lim = src ? (uint32_t)(SPARSE ? L.off_w2 + H * H * L.es : L.off_w2) : 0u;
+  }
+  // Copy the next batch into the ring's place at `pos` and step on.
+  __device__ __forceinline__ void copy(const Layout &L, int lane) {
+#pragma unroll
+    for (int k = 0; k < UB; ++k)
+      if (off + 512u * k < lim)
+        asm volatile("cp.async.cg.shared.global.L2::256B [%0], [%1], 16;" ::"r"(lane0 + pos + 512u * k),
+                     "l"(src + off + 512u * k)
+                     : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    pos = pos + 512u * UB == kBytes ? 0u : pos + 512u * UB;
+    off += 512u * UB;
+    if (--left == 0) {
+      ++sec;
+      if (sec > L.L + 1) {
+        src = nxt;
+        nxt = nullptr;
+        start(L, lane);
+      } else if (sec == L.L + 1) {
+        off = (uint32_t)L.off_w3 + 16u * (uint32_t)lane;
+        lim = src ? (uint32_t)(L.off_w3 + L.A * H * L.es) : 0u;
+        left = ring_batches(L.A * UPJ, UB);
+      } else {
+        off = (uint32_t)(L.off_w2 + (sec - 1) * H * H * L.es) + 16u * (uint32_t)lane;
+        lim = src ? (uint32_t)(L.off_w2 + sec * H * H * L.es) : 0u;
+        left = ring_batches(H * UPJ, UB);
+      }
+    }
+  }
+  __device__ __forceinline__ void read(uint4 *v) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(NB - 1) : "memory");
+#pragma unroll
+    for (int k = 0; k < UB; ++k) v[k] = lds_unit(lane0 + pos + 512u * k);
+  }
+};
+
+// One input-major layer from the ring.
+template <int PREC, int H, int NB, int UB, bool SPARSE>
+__device__ __forceinline__ void ring_layer(Ring<PREC, H, NB, UB, SPARSE> &ring, const Layout &L, int n_in,
+                                           const float *__restrict__ x, const float *__restrict__ bias, int nbias,
+                                           const float *__restrict__ scale, float *__restrict__ out, int lane,
+                                           int n_exact) {
+  constexpr int E = Unit<PREC>::E;
+  constexpr int UPJ = H / E;
+  constexpr int LG = Log2<UPJ>::v;
+  constexpr int NOUT = H / 32;
+  // this lane's bias and scale, requested before the stream and used after it
+  const int o0 = finish_first<PREC, H>(lane);
+  float b[NOUT], sc[NOUT];
+#pragma unroll
+  for (int i = 0; i < NOUT; ++i) {
+    sc[i] = (PREC == PREC_FP8) ? __ldg(scale + o0 + i) : 1.0f;
+    b[i] = __ldg(bias + o0 + i);
+    for (int k = 1; k < nbias; ++k) b[i] += __ldg(bias + k * H + o0 + i);
+  }
+  float acc[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) acc[e] = 0.0f;
+  const int U = n_in * UPJ;
+  const int U_h = PREC == PREC_FP8 ? n_exact * UPJ : 0;
+  int u = lane;
+#pragma unroll 1
+  for (int r0 = 0; r0 < U; r0 += 32 * UB, u += 32 * UB) {
+    uint4 v[UB];
+    ring.read(v);
+    if (PREC == PREC_FP8 && r0 + 32 * UB <= U_h) {
+      if constexpr (PREC == PREC_FP8) {
+#pragma unroll
+        for (int k = 0; k < UB; ++k)
+          Unit<PREC>::fma_h(acc, v[k], __half_as_ushort(__float2half_rn(x[(u + 32 * k) >> LG])));
+      }
+    } else if (r0 + 32 * UB <= U) {
+#pragma unroll
+      for (int k = 0; k < UB; ++k) Unit<PREC>::fma(acc, v[k], x[(u + 32 * k) >> LG]);
+    } else {  // the layer's last units; the rest of v was not copied
+#pragma unroll
+      for (int k = 0; k < UB; ++k)
+        if (u + 32 * k < U) Unit<PREC>::fma(acc, v[k], x[(u + 32 * k) >> LG]);
+    }
+    ring.copy(L, lane);
+  }
+  finish_sums<PREC, H>(acc, lane);
+#pragma unroll
+  for (int i = 0; i < NOUT; ++i) {
+    const float v = fmaf(acc[i], sc[i], b[i]);
+    out[o0 + i] = L.relu ? fmaxf(v, 0.0f) : tanhf(v);
+  }
+}
+
+template <int PREC, int H, int WARPS, int MINB, int NB, int UB, bool SPARSE>
+__global__ void __launch_bounds__(WARPS * 32, MINB)
+    k_policy_ring(Dev d, Layout L, Rules R, int xs_floats, int apply_moves) {
+  constexpr int E = Unit<PREC>::E;
+  constexpr int UPJ = H / E;
+  typedef Ring<PREC, H, NB, UB, SPARSE> RingT;
+  extern __shared__ __align__(128) unsigned char ring_smem[];
+  const int lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5;
+  float *xs = reinterpret_cast<float *>(ring_smem + WARPS * RingT::kBytes) +
+              warp * policy_warp_floats(xs_floats, H, SPARSE);
+  float *hs = xs + xs_floats;
+  float *ls = hs + H;
+
+  const int n_alive = d.counters[CNT_N_ALIVE];
+  const uint32_t t = (uint32_t)d.step[0];
+  const int w0 = blockIdx.x * WARPS + warp;
+  // the list has total_slots entries: in bounds even past the count
+  int slot_n = w0 < d.total_slots ? d.alive_list[w0] : 0;
+  if (apply_moves && blockIdx.x == 0 && threadIdx.x == 0) d.alive_at_step[t & (kAliveRing - 1)] = n_alive;
+  const int G = gridDim.x * WARPS;
+  const int rounds = (n_alive + G - 1) / G;
+  const int G_eff = rounds > 0 ? (n_alive + rounds - 1) / rounds : G;
+  if (w0 >= G_eff || w0 >= n_alive) return;
+
+  RingT ring;
+  ring.lane0 = smem_addr(ring_smem) + (uint32_t)warp * RingT::kBytes + 16u * (uint32_t)lane;
+  ring.pos = 0u;
+  ring.src = d.wq + (int64_t)slot_n * L.stride;
+  ring.nxt = nullptr;
+  ring.start(L, lane);
+  // an agent has NB batches at least, so the ring reaches into the next
+  // agent's block at most
+#pragma unroll 1
+  for (int b = 0; b < NB; ++b) ring.copy(L, lane);
+
+  const int k = R.patch_k;
+  const uint32_t kdiv = k > 0 ? 0xFFFFFFFFu / (uint32_t)k + 1u : 0u;
+  const bool greedy = (R.flags & F_GREEDY) != 0;
+  int cnt = 0, e_cur = -1;
+  auto flush = [&]() {
+    if (e_cur >= 0 && cnt && lane <= 16)
+      atomicAdd((unsigned long long *)&d.stats_step[e_cur * N_ST + (lane < 16 ? ST_ACT0 + lane : ST_MOVE_BLOCKED)],
+                (unsigned long long)cnt);
+    cnt = 0;
+  };
+  // one-hot vision under the simple rules: the next agent's cells are read
+  // while the current agent's head and sampling run
+  const bool ahead = R.vision == VISION_CHANNELS && R.rules == RULES_SIMPLE && k * k <= 32 * kCellsAhead;
+  CellsAhead ca;
+  int env_n = d.env_of[slot_n], pos_n = d.pos[slot_n], f_n = d.facing[slot_n];
+  if (ahead) cells_load(d, R, slot_n, env_n, pos_n, f_n, lane, kdiv, ca);
+  for (int i = w0; i < n_alive; i += G_eff) {
+    const int slot = slot_n, env = env_n, pos = pos_n, f = f_n;
+    const bool more = i + G_eff < n_alive;
+    if (more) slot_n = d.alive_list[i + G_eff];
+    if (env != e_cur) {
+      flush();
+      e_cur = env;
+    }
+    int nb_cell = 0;
+    uint32_t nb_flags = 0;
+    short *idx = reinterpret_cast<short *>(ls + 16);
+    int n_nz = 0;
+    if (ahead) {
+      if constexpr (SPARSE) n_nz = cells_list(R, ca, f, xs, idx, lane);
+      else cells_store(R, L, ca, f, xs, lane);
+      nb_cell = ca.nb_cell;
+      nb_flags = ca.nb_flags;
+    } else {
+      gather_obs(d, L, R, slot, env, pos, f, xs, lane, kdiv, &nb_cell, &nb_flags);
+      if constexpr (SPARSE) {
+        __syncwarp();
+        n_nz = list_nonzero(L.D, xs, idx, lane);
+      }
+    }
+    __syncwarp();
+    ring.nxt = more ? d.wq + (int64_t)slot_n * L.stride : nullptr;
+
+    const uint8_t *blk = d.wq + (int64_t)slot * L.stride;
+    const float *bias = reinterpret_cast<const float *>(blk + L.off_bias);
+    const float *scale = reinterpret_cast<const float *>(blk + L.off_scale);
+    if constexpr (SPARSE) {
+      layer_in_major<PREC, H, 8, true>(reinterpret_cast<const uint4 *>(blk), n_nz, xs, bias, L.ns, scale, hs, lane,
+                                       L.relu, idx);
+    } else {
+      // one-hot vision: the patch inputs are 0 or 1, exact in f16
+      ring_layer<PREC, H, NB, UB, SPARSE>(ring, L, L.D, xs, bias, L.ns, scale, hs, lane,
+                                          R.vision == VISION_CHANNELS ? L.patch : 0);
+    }
+    if (more) {
+      env_n = d.env_of[slot_n];
+      pos_n = d.pos[slot_n];
+      f_n = d.facing[slot_n];
+    }
+    __syncwarp();
+    float *cur = hs, *nxt = xs;
+    for (int l = 0; l < L.L; ++l) {
+      ring_layer<PREC, H, NB, UB, SPARSE>(ring, L, H, cur, bias + L.ns * H + l * H, 1, scale + H + l * H, nxt, lane, 0);
+      __syncwarp();
+      float *tmp = cur;
+      cur = nxt;
+      nxt = tmp;
+    }
+    if (more && ahead) cells_load(d, R, slot_n, env_n, pos_n, f_n, lane, kdiv, ca);
+    const int U3 = L.A * UPJ;
+    const float *hb = bias + L.ns * H + L.L * H;  // head bias, then tau
+    const float tmul = L.temp ? expf(-__ldg(hb + (L.out_bias ? L.A : 0))) : 1.0f;
+    for (int base = 0; base < U3; base += 32 * UB) {
+      uint4 v[UB];
+      ring.read(v);
+#pragma unroll
+      for (int g = 0; g < UB; ++g)
+        if (base + 32 * g < U3)
+          head_group<PREC, H>(v[g], base + 32 * g + lane, U3, cur, scale + H + L.L * H, hb, L.out_bias, L.temp, tmul, ls,
+                              lane);
+      ring.copy(L, lane);
+    }
+    __syncwarp();
+    sample_and_claim(d, R, L.A, slot, env, pos, f, ls, lane, t, greedy, apply_moves, nb_cell, nb_flags, cnt);
+    __syncwarp();
+  }
+  flush();
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// ---------------------------------------------------------------------------
 // Variant k (1-based) of one precision and hidden width.  Variants 7 and 8
 // are the input-sparse forms of 3 and 6 (they stream only the W_in rows of
 // nonzero inputs); the autotuner keeps the two families apart.  Variants 9
 // and 10 sit between the 48- and 64-register ones: 56 registers, 36 warps
-// per SM.
+// per SM.  Variants 3 and 7 are the ring form: 20 warps per SM at 96
+// registers, 16 rows (8 KB) in flight per warp.  Other splits of an SM's
+// shared memory measured on 371-64-64-9 FP8 at 12,000 and 48,000 agents:
+// this one 63 and 212 us, 24 warps x 12 rows 64 and 223, 16 warps x 20 rows
+// 64 and 214, 28 warps x 8 rows 72 and 257.
 // ---------------------------------------------------------------------------
 template <int PREC, int H>
 PolicyFn policy_pick_variant(int variant) {
   switch (variant) {
     case 1: return k_policy<PREC, H, 4, 8, 10, false>;
     case 2: return k_policy<PREC, H, 8, 8, 5, false>;
-    case 3: return k_policy<PREC, H, 8, 4, 5, false>;
+    case 3: return k_policy_ring<PREC, H, 4, 5, 4, 4, false>;
     case 4: return k_policy<PREC, H, 16, 4, 2, false>;
     case 5: return k_policy<PREC, H, 8, 4, 4, false>;
     case 6: return k_policy<PREC, H, 4, 8, 8, false>;
-    case 7: return k_policy<PREC, H, 8, 4, 5, true>;
+    case 7: return k_policy_ring<PREC, H, 4, 5, 4, 4, true>;
     case 8: return k_policy<PREC, H, 4, 8, 8, true>;
     case 9: return k_policy<PREC, H, 4, 8, 9, false>;
     case 10: return k_policy<PREC, H, 4, 4, 9, false>;
