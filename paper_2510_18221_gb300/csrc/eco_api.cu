@@ -61,6 +61,7 @@ struct eco_handle {
   // steps run since reset (a host shadow of the device's step counter) and
   // the first step of every timed launch not yet reported
   long long steps_done;
+  bool list_current;  // the alive list is that of the current state
   std::vector<long long> timed_steps;
   cudaEvent_t ev_dummy[2];
   std::vector<cudaEvent_t> ev_pool;  // pairs
@@ -468,6 +469,7 @@ extern "C" int eco_create(const eco_config *cfg, void *dev_workspace, size_t byt
   }
   h->ev_used = 0;
   h->steps_done = 0;
+  h->list_current = false;
   h->rd_pending = 0;
   h->rd_ev[0] = h->rd_ev[1] = nullptr;
   h->err[0] = 0;
@@ -542,13 +544,25 @@ static int check_status(eco_handle *h) {
   return ECO_OK;
 }
 
+// The alive list of the current state.  Reset, state writes and every step
+// leave it so: only a handle that has seen none of them still has to make it
+// (eco_policy_only made it on each call, two kernels of 2 us).
+static int make_list(eco_handle *h) {
+  if (h->list_current) return ECO_OK;
+  CUDA_TRY(h, launch_compact(h->d, h->stream));
+  h->list_current = true;
+  return ECO_OK;
+}
+
 extern "C" int eco_reset(eco_handle *h) {
   if (!h) return fail(nullptr, ECO_EINVAL, "null handle");
   // also clears the status word, the persistent form's barrier and its
   // failure-detection test words
   CUDA_TRY(h, cudaMemsetAsync(h->d.barrier, 0, BAR_N * sizeof(unsigned), h->stream));
+  h->list_current = false;
   CUDA_TRY(h, launch_reset(h->d, h->L, h->R, h->grid, h->stream));
-  CUDA_TRY(h, launch_compact(h->d, h->stream));
+  const int rc = make_list(h);
+  if (rc) return rc;
   h->rd_pending = 0;  // eco_step_read starts over from the reset records
   h->steps_done = 0;
   return check_status(h);
@@ -571,7 +585,8 @@ extern "C" int eco_reset_seed(eco_handle *h, uint64_t seed) {
 // Choose the fastest policy variant on the current state (autotuner).
 static int autotune(eco_handle *h) {
   if (h->variant) return ECO_OK;
-  CUDA_TRY(h, launch_compact(h->d, h->stream));
+  int rc = make_list(h);
+  if (rc) return rc;
   // candidates of the requested family
   const bool sparse = h->forced < 0;
   std::vector<int> ids;
@@ -790,8 +805,8 @@ extern "C" int eco_policy_timing(eco_handle *h, double *total_ms, int32_t *n_tim
 extern "C" int eco_policy_only(eco_handle *h, int32_t n_iters) {
   if (!h) return fail(nullptr, ECO_EINVAL, "null handle");
   int rc = autotune(h);
+  if (rc == ECO_OK) rc = make_list(h);
   if (rc) return rc;
-  CUDA_TRY(h, launch_compact(h->d, h->stream));
   for (int i = 0; i < n_iters; ++i) CUDA_TRY(h, policy_launch(h->pl, h->d, h->L, h->R, h->stream, false));
   return ECO_OK;
 }
@@ -849,7 +864,8 @@ extern "C" int eco_launch_mode(const eco_handle *h, int32_t *mode, int32_t *bloc
 extern "C" int eco_policy_bytes(eco_handle *h, int64_t *bytes, int64_t *n_alive) {
   if (!h) return fail(nullptr, ECO_EINVAL, "null handle");
   int32_t n = 0;
-  CUDA_TRY(h, launch_compact(h->d, h->stream));
+  int rc = make_list(h);
+  if (rc) return rc;
   CUDA_TRY(h, cudaMemcpyAsync(&n, h->d.counters + CNT_N_ALIVE, sizeof n, cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
   const Layout &L = h->L;
@@ -871,7 +887,10 @@ static int stats_from_mirror(eco_handle *h, int slot, eco_stats *total, eco_stat
   int32_t st = 0;
   memcpy(&st, mirror(h->d.counters + CNT_STATUS), sizeof st);
   if (st & 3) return fail(h, ECO_EINVAL, "reset: fewer non-wall cells than founders (status %d)", st);
-  if (st & 4) return fail(h, ECO_ETIMEOUT, "a device-side wait ran out of its budget");
+  if (st & 4) {
+    h->list_current = false;  // the state is partly stepped
+    return fail(h, ECO_ETIMEOUT, "a device-side wait ran out of its budget");
+  }
   return ECO_OK;
 }
 
@@ -1012,6 +1031,7 @@ extern "C" int eco_write_state(eco_handle *h, int32_t env, const eco_state_view 
         return fail(h, ECO_EINVAL, "slot %d position out of range", i);
       pos[i] = in->y[i] * ed.side + in->x[i];
     }
+    h->list_current = false;
     CUDA_TRY(h, cudaMemcpyAsync(h->d.alive + ed.slot_off, alive.data(), S, cudaMemcpyHostToDevice, s));
     CUDA_TRY(h, cudaMemcpyAsync(h->d.pos + ed.slot_off, pos.data(), 4 * (size_t)S, cudaMemcpyHostToDevice, s));
   }
@@ -1059,7 +1079,9 @@ extern "C" int eco_write_state(eco_handle *h, int32_t env, const eco_state_view 
     CUDA_TRY(h, cudaStreamSynchronize(s));
   }
   CUDA_TRY(h, launch_recount(h->d, h->R, s));
-  CUDA_TRY(h, launch_compact(h->d, s));
+  h->list_current = false;
+  rc = make_list(h);
+  if (rc) return rc;
   // the persistent form's arrival counts are kept per step parity, which a
   // written step may change: both start from zero
   CUDA_TRY(h, cudaMemsetAsync(h->d.barrier + BAR_COUNT0, 0, 2 * sizeof(unsigned), s));
