@@ -51,8 +51,8 @@ struct eco_handle {
   // kStepsPerGraph steps (eco_step).  An event-record node costs a few us
   // on the critical path between two kernels, so the untimed graphs have
   // none, and a graph of several steps saves the launch gap between graphs.
-  // [GRAPH_READ1], [GRAPH_READ2]: one step, then a copy of the statistics
-  // into pinned slot 1 or 2 (eco_step_read); [GRAPH_TIMED_MANY]:
+  // [GRAPH_READ1], [GRAPH_READ2]: one step that leaves its records in pinned
+  // slot 1 or 2 (eco_step_read); [GRAPH_TIMED_MANY]:
   // kStepsPerGraph steps with event-record nodes around the first step's
   // policy kernel only (eco_step_timed: one timed launch per graph)
   cudaGraphExec_t graph[6];
@@ -642,14 +642,22 @@ static int autotune(eco_handle *h) {
 // write_state), so the step is the policy kernel and the environment
 // phases, which end by building the next step's alive list.  timed: an
 // event-record node on each side of the policy kernel.
-static cudaError_t enqueue_step(eco_handle *h, bool timed) {
+// mirror: pinned memory that receives the step's records and status word
+// (the persistent form writes them itself, where a copy node behind the step
+// took 3 us of the GPU; the per-phase form ends with the copy), or null.
+static cudaError_t enqueue_step(eco_handle *h, bool timed, uint8_t *mirror) {
   cudaError_t e = cudaSuccess;
   // "external" records become event-record nodes of the captured graph
   if (timed) e = cudaEventRecordWithFlags(h->ev_dummy[0], h->stream, cudaEventRecordExternal);
   if (e == cudaSuccess) e = policy_launch(h->pl, h->d, h->L, h->R, h->stream, true);
   if (e == cudaSuccess && timed)
     e = cudaEventRecordWithFlags(h->ev_dummy[1], h->stream, cudaEventRecordExternal);
-  if (e == cudaSuccess) e = launch_env_phases(h->d, h->L, h->R, h->grid, h->stream);
+  const bool persistent = h->grid.use_persistent && h->grid.persistent_blocks > 0;
+  Dev d = h->d;
+  if (persistent) d.mirror = mirror;
+  if (e == cudaSuccess) e = launch_env_phases(d, h->L, h->R, h->grid, h->stream);
+  if (e == cudaSuccess && mirror && !persistent)
+    e = cudaMemcpyAsync(mirror, h->d.stats_total, h->rd_bytes, cudaMemcpyDeviceToHost, h->stream);
   return e;
 }
 
@@ -664,10 +672,7 @@ static int build_graph(eco_handle *h, int kind) {
   for (;;) {
     CUDA_TRY(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
-    for (int k = 0; k < steps && e == cudaSuccess; ++k) e = enqueue_step(h, timed && k == 0);
-    if (e == cudaSuccess && copy_slot)
-      e = cudaMemcpyAsync(h->rd_host + copy_slot * h->rd_bytes, h->d.stats_total, h->rd_bytes,
-                          cudaMemcpyDeviceToHost, h->stream);
+    for (int k = 0; k < steps && e == cudaSuccess; ++k) e = enqueue_step(h, timed && k == 0, copy_slot ? h->rd_host + copy_slot * h->rd_bytes : nullptr);
     cudaError_t e2 = cudaStreamEndCapture(h->stream, &g);
     if (e == cudaSuccess && e2 == cudaSuccess) break;
     if (e2 == cudaSuccess && g) cudaGraphDestroy(g);

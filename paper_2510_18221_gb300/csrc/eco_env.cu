@@ -1339,7 +1339,8 @@ __device__ void fold_env(const Dev &d, const Rules &R, int e, long long t, int b
   for (int q = 0; q < 2; ++q) {
     const int k = lane + 32 * q;
     if (k >= N_ST) break;
-    long long v = o[q], l;
+    long long v = o[q], l = 0;
+    bool is_sum = false;
     if (k == ST_STEP) {
       v = t + 1;
     } else if (k == ST_ALIVE) {
@@ -1357,15 +1358,19 @@ __device__ void fold_env(const Dev &d, const Rules &R, int e, long long t, int b
       v += k == ST_BIO_CELLS ? bio : -bio;
     } else {
       l = k == ST_AGENT_STEPS ? as : k == ST_ATTACKS ? attacks : s[q];
-      last[k] = l;
-      tot[k] = v + l;
-      st[k] = 0;
-      continue;
+      v += l;
+      is_sum = true;
     }
-    last[k] = v;
+    if (!is_sum) l = v;
+    last[k] = l;
     tot[k] = v;
     st[k] = 0;
+    if (d.mirror) {
+      *mirror_of(d, last + k) = l;
+      *mirror_of(d, tot + k) = v;
+    }
   }
+  if (d.mirror && e == 0 && lane == 0) *mirror_of(d, d.counters + CNT_STATUS) = d.counters[CNT_STATUS];
 }
 
 // ---------------------------------------------------------------------------
@@ -1628,7 +1633,16 @@ __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rul
                  cuda::memory_order_relaxed) & kStatusTimeout;
   }
   __syncthreads();
-  if (s_flag) return;
+  if (s_flag) {
+    // the host's copy, which no fold will write: everything as it stands
+    if (d.mirror && blockIdx.x == 0) {
+      const int words = (int)(reinterpret_cast<const int32_t *>(d.counters + CNT_N) -
+                              reinterpret_cast<const int32_t *>(d.stats_total));
+      for (int i = threadIdx.x; i < words; i += blockDim.x)
+        reinterpret_cast<int32_t *>(d.mirror)[i] = reinterpret_cast<const int32_t *>(d.stats_total)[i];
+    }
+    return;
+  }
   if (absent == blockIdx.x + 1u) return;
   const unsigned budget = budget_word ? budget_word : kBarrierSpinLimit;
   unsigned *count = d.barrier + BAR_COUNT0 + (t & 1u);
@@ -1650,6 +1664,7 @@ __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rul
       if (threadIdx.x == 0) atomicMax(trow + TR_ARRIVE0 + bar, global_ns());
     }
     const bool ok = grid_sync(count, d.counters + CNT_STATUS, nb, budget, bar, &s_flag);
+    if (!ok && d.mirror && threadIdx.x == 0) *mirror_of(d, d.counters + CNT_STATUS) = kStatusTimeout;
     if (trow && blockIdx.x == 0 && threadIdx.x == 0) trow[TR_PASS0 + bar - 1] = global_ns();
     return ok;
   };

@@ -323,7 +323,17 @@ struct Dev {
   uint32_t *flow;          // [total_cells] this step's transfer: amount << 2 | direction
   int32_t *a_water;        // [total_slots] water carried
   int32_t *a_bio;          // [total_slots] biomass carried
+  // The host's copy of the records (pinned, null: none), laid out as the
+  // workspace from stats_total through counters: the persistent form writes
+  // the step's records and status word there itself (eco_step_read).
+  uint8_t *mirror;
 };
+
+template <class T>
+__device__ __forceinline__ T *mirror_of(const Dev &d, const T *p) {
+  return reinterpret_cast<T *>(d.mirror + (reinterpret_cast<const uint8_t *>(p) -
+                                           reinterpret_cast<const uint8_t *>(d.stats_total)));
+}
 
 constexpr int kAliveRing = 4096;
 // Readable workspace bytes after the last slot's weight block: the policy
