@@ -1499,88 +1499,61 @@ __device__ void list_free_slots(const Dev &d, int *sh) {
 // The fast birth path (one environment, at most kFastBirths claimants):
 // every CTA derives the same births from the claims and the free-slot list
 // (written in the birth-claim phase, when the deaths were final), so no
-// barrier separates the slot assignment
-// from the mutation and the alive list: pair i is (S.win[i], S.free_[i]),
-// i < S.nborn, of S.nwin winners.
+// barrier separates the slot assignment from the mutation and the alive
+// list: pair i is (S.win[i], S.free_[i]), i < S.nborn, of S.nwin winners.  A
+// thread per claimant ranks its winner by comparison with all the others
+// (sorting them took a block barrier per exchange); a warp adds up the
+// tiles' free slots meanwhile.
 __device__ void fast_births(const Dev &d, BirthSmem &S, int nc) {
   const EnvDesc ed = d.env[0];
-  // The first nc free slots (at most nc are needed), read with the claims
-  // rather than after the sort: from the per-tile lists of list_free_slots,
-  // tile k's entries covering ranks [before_k, before_k + min(free_k, cap)).
+  const int tid = threadIdx.x, lane = tid & 31;
+  int *const key = S.win + kBirthCap / 2;  // winners' slots, claimant by claimant
+  static_assert(2 * kFastBirths <= kBirthCap, "the keys and the ranked winners share an array");
+  int g = 0x7FFFFFFF;
+  if (tid < nc) {
+    const int c = d.contenders[ed.slot_off + tid];
+    const int bt = d.bcell[ed.slot_off + tid];
+    if (claim_local_slot(d.claim_birth[ed.cell_off + bt]) == c - ed.slot_off) g = c;
+    key[tid] = g;
+  }
   const int tiles = (ed.n_slots + kCompactTile - 1) / kCompactTile;
-  if (threadIdx.x == 0) {
-    int before = 0;
-    for (int k = 0; k < tiles; ++k) {
-      S.tile_first[k] = before;
-      before += d.free_tiles[k];
-    }
-    S.nfree = before;
-  }
-  __syncthreads();
-  const int want = nc < S.nfree ? nc : S.nfree;
-  for (int i = threadIdx.x; i < want; i += blockDim.x) {
-    int k = 0;
-    while (k + 1 < tiles && S.tile_first[k + 1] <= i) ++k;
-    S.free_[i] = ed.slot_off + d.free_list[k * kFastBirths + (i - S.tile_first[k])];
-  }
-  const int nwin = sort_winners(d, ed, nc, S);  // synchronises the CTA
-  const int nborn = nwin < S.nfree ? nwin : S.nfree;
-  if (threadIdx.x == 0) S.nborn = nborn;
-  __syncthreads();
-}
-
-// fast_births for at most 32 claimants, by the CTA's first warp: a lane per
-// claimant, ranks by comparison, no block barrier but the last (the sort's
-// and the scan's were most of the path's time).
-__device__ void fast_births_few(const Dev &d, BirthSmem &S, int nc) {
-  if (threadIdx.x < 32) {
-    const EnvDesc ed = d.env[0];
-    const int lane = threadIdx.x;
-    const int g = lane < nc ? d.contenders[ed.slot_off + lane] : 0x7FFFFFFF;
-    const int bt = lane < nc ? d.bcell[ed.slot_off + lane] : 0;
-    // free slots before each tile: eight tiles per lane
+  if (tid >= (int)blockDim.x - 32) {  // free slots before each tile: eight tiles per lane
     constexpr int kPer = kMaxFastTiles / 32;
-    const int tiles = (ed.n_slots + kCompactTile - 1) / kCompactTile;
     int f[kPer], own = 0;
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
       f[k] = lane * kPer + k < tiles ? d.free_tiles[lane * kPer + k] : 0;
       own += f[k];
     }
-    const bool won = lane < nc && claim_local_slot(d.claim_birth[ed.cell_off + bt]) == g - ed.slot_off;
     int incl = own;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
       const int o = __shfl_up_sync(0xFFFFFFFFu, incl, off);
       if (lane >= off) incl += o;
     }
-    const int nfree = __shfl_sync(0xFFFFFFFFu, incl, 31);
     int before = incl - own;
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
       S.tile_first[lane * kPer + k] = before;
       before += f[k];
     }
+    if (lane == 31) S.nfree = incl;
+  }
+  const int nwin = __syncthreads_count(g != 0x7FFFFFFF);
+  const int nfree = S.nfree, nborn = nwin < nfree ? nwin : nfree;
+  if (g != 0x7FFFFFFF && nborn > 0) {
     int rank = 0;
-#pragma unroll
-    for (int l = 0; l < 32; ++l) {
-      const int o = __shfl_sync(0xFFFFFFFFu, won ? g : 0x7FFFFFFF, l);
-      rank += o < g ? 1 : 0;
-    }
-    const int nwin = __popc(__ballot_sync(0xFFFFFFFFu, won));
-    if (won) S.win[rank] = g;
-    __syncwarp();
-    const int nborn = nwin < nfree ? nwin : nfree;
-    if (lane < nborn) {
-      int k = 0;
-      while (k + 1 < tiles && S.tile_first[k + 1] <= lane) ++k;
-      S.free_[lane] = ed.slot_off + d.free_list[k * kFastBirths + (lane - S.tile_first[k])];
-    }
-    if (lane == 0) {
-      S.nwin = nwin;
-      S.nfree = nfree;
-      S.nborn = nborn;
-    }
+    for (int i = 0; i < nc; ++i) rank += key[i] < g ? 1 : 0;
+    S.win[rank] = g;
+  }
+  if (tid < nborn) {
+    int k = 0;
+    while (k + 1 < tiles && S.tile_first[k + 1] <= tid) ++k;
+    S.free_[tid] = ed.slot_off + d.free_list[k * kFastBirths + (tid - S.tile_first[k])];
+  }
+  if (tid == 0) {
+    S.nwin = nwin;
+    S.nborn = nborn;
   }
   __syncthreads();
 }
@@ -1604,6 +1577,9 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return v;
 }
 
+// CLUSTER: the grid is one thread-block cluster, whose hardware barrier takes
+// the grid barrier's place.
+template <bool CLUSTER>
 __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rules R) {
   extern __shared__ __align__(16) float msm[];
   __shared__ BirthSmem S;
@@ -1663,7 +1639,14 @@ __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rul
       __syncthreads();
       if (threadIdx.x == 0) atomicMax(trow + TR_ARRIVE0 + bar, global_ns());
     }
-    const bool ok = grid_sync(count, d.counters + CNT_STATUS, nb, budget, bar, &s_flag);
+    bool ok = true;
+    if constexpr (CLUSTER) {
+      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+      ++bar;
+    } else {
+      ok = grid_sync(count, d.counters + CNT_STATUS, nb, budget, bar, &s_flag);
+    }
     if (!ok && d.mirror && threadIdx.x == 0) *mirror_of(d, d.counters + CNT_STATUS) = kStatusTimeout;
     if (trow && blockIdx.x == 0 && threadIdx.x == 0) trow[TR_PASS0 + bar - 1] = global_ns();
     return ok;
@@ -1671,9 +1654,14 @@ __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rul
   // Housekeeping goes to CTAs with little else to do in its interval: the
   // per-agent phases take one agent per thread from CTA 0 on, and the
   // alive list's tiles go to CTAs 0 .. tiles - 1.  The cells' phases leave
-  // the CTAs with agents out where those are at most half.
+  // the CTAs with agents out where those are at most half and the others
+  // have at most four groups a thread (a 2048 x 2048 world or a large batch
+  // has more, and needs every SM).
   const int agent_ctas = (n_alive + (int)blockDim.x - 1) / (int)blockDim.x;
-  const int cell_first = agent_ctas * 2 <= (int)nb ? agent_ctas : 0;
+  const int rest = (int)nb - agent_ctas;
+  const int cell_first =
+      rest >= agent_ctas && (d.total_cells >> 2) <= 4ll * rest * (int)blockDim.x ? agent_ctas : 0;
+  const int regrow_ahead = cell_first > 0 && d.n_envs == 1 ? kRegrowAhead : 0;
   const int cg0 = g0 - cell_first * (int)blockDim.x, cgs = gs - cell_first * (int)blockDim.x;
   const bool cell_cta = (int)blockIdx.x >= cell_first;
   const int tiles = compact_tiles(d.total_slots);
@@ -1693,7 +1681,7 @@ __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rul
   ph_move_apply_eat(d, R, L.A, g0, gs, first, t, ag);
   if (cell_cta) {
     if (R.rules != RULES_TERRAIN) {
-      draws = regrow_draws(d, R, cg0, cgs, t);
+      if (regrow_ahead) draws = regrow_draws(d, R, cg0, cgs, t);
     } else {
       // the policy kernel's weight stream has pushed the cells' planes out of
       // L2: bring them back ahead of the cells' phases
@@ -1709,7 +1697,7 @@ __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rul
   if (!sync()) return;
   ph_metab_death(d, R, g0, gs, t, ag);
   // simple rules: only eating takes food, and it is over
-  if (R.rules == RULES_SIMPLE && cell_cta) ph_regrow(d, R, cg0, cgs, t, draws, kRegrowAhead);
+  if (R.rules == RULES_SIMPLE && cell_cta) ph_regrow(d, R, cg0, cgs, t, draws, regrow_ahead);
   if (!sync()) return;
   // regrowth under the other rules (with photosynthesis and the flow's
   // transfers) needs the state after the deaths, and birth claims read only
@@ -1719,7 +1707,7 @@ __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rul
   if (d.n_envs == 1 && compact_tiles(d.total_slots) <= kMaxFastTiles) list_free_slots(d, S.sh);
   TileScan ts = {0u, 0, 0, 0};
   if (tiles <= (int)nb && (int)blockIdx.x < tiles) ts = compact_scan(d, blockIdx.x, S.sh64, t);
-  if (R.rules != RULES_SIMPLE && cell_cta) ph_regrow(d, R, cg0, cgs, t, draws, kRegrowAhead);
+  if (R.rules != RULES_SIMPLE && cell_cta) ph_regrow(d, R, cg0, cgs, t, draws, regrow_ahead);
   if (R.rules == RULES_TERRAIN && cell_cta) ph_flow_out(d, cg0, cgs);
   if (!sync()) return;
   // Every claim is in, and the count of claimants does not change again
@@ -1734,8 +1722,7 @@ __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rul
     ph_birth_assign(d, R, blockIdx.x, gridDim.x, S, t);
     if (!sync()) return;
   } else if (fast) {
-    if (claimants <= 32) fast_births_few(d, S, claimants);
-    else fast_births(d, S, claimants);
+    fast_births(d, S, claimants);
   }
   // Every statistic of the step is in: one CTA folds them, a warp per
   // environment from its last warp on, while the others go on.
@@ -1800,18 +1787,52 @@ cudaError_t env_prepare(const Layout &L, EnvGrid *g) {
   cudaError_t e = cudaFuncSetAttribute((const void *)k_mutate, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute((const void *)k_env_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem);
-  if (e != cudaSuccess) return e;
+  const void *const forms[2] = {(const void *)k_env_persistent<false>, (const void *)k_env_persistent<true>};
+  for (const void *f : forms)
+    if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
   int dev = 0, coop = 0, per_sm = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)k_env_persistent, 1024,
-                                                         smem)) != cudaSuccess)
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, forms[0], 1024, smem)) != cudaSuccess)
     return e;
   // one CTA per SM: fewer arrivals on the barrier counter
   g->persistent_blocks = (coop && per_sm >= 1) ? g->sms : 0;
+  g->cluster = 0;
   return cudaSuccess;
+}
+
+// A small batch's persistent form: one cluster of kSmallCluster CTAs, or one
+// CTA where the device offers none of that size.
+constexpr int kSmallCluster = 8;
+
+static cudaLaunchConfig_t persistent_config(const Layout &L, int blocks, bool cluster, cudaStream_t s,
+                                            cudaLaunchAttribute *attr) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(1024);
+  cfg.dynamicSmemBytes = mutate_smem_bytes(L);
+  cfg.stream = s;
+  if (cluster) {
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = (unsigned)blocks;
+    attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+  } else {
+    attr->id = cudaLaunchAttributeCooperative;
+    attr->val.cooperative = 1;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+void env_use_small_grid(const Layout &L, EnvGrid *g) {
+  cudaLaunchAttribute attr;
+  const cudaLaunchConfig_t cfg = persistent_config(L, kSmallCluster, true, nullptr, &attr);
+  int clusters = 0;
+  const cudaError_t e = cudaOccupancyMaxActiveClusters(&clusters, (const void *)k_env_persistent<true>, &cfg);
+  if (e != cudaSuccess) cudaGetLastError();
+  g->cluster = e == cudaSuccess && clusters > 0;
+  g->persistent_blocks = g->cluster ? kSmallCluster : 1;
 }
 
 // The step's phases after the policy kernel, ending with the alive list of
@@ -1820,17 +1841,10 @@ cudaError_t launch_env_phases(const Dev &d, const Layout &L, const Rules &R, con
                               cudaStream_t s) {
   const size_t msmem = mutate_smem_bytes(L);
   if (g.persistent_blocks > 0 && g.use_persistent) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(g.persistent_blocks);
-    cfg.blockDim = dim3(1024);
-    cfg.dynamicSmemBytes = msmem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_env_persistent, d, L, R);
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = persistent_config(L, g.persistent_blocks, g.cluster != 0, s, &attr);
+    return g.cluster ? cudaLaunchKernelEx(&cfg, k_env_persistent<true>, d, L, R)
+                     : cudaLaunchKernelEx(&cfg, k_env_persistent<false>, d, L, R);
   }
   const int T = 256;
   k_move_apply_eat<<<g.slot_blocks, T, 0, s>>>(d, R, L.A);

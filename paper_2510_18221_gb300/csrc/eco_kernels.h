@@ -47,12 +47,15 @@ struct EnvGrid {
   int birth_blocks;       // CTAs of the mutation kernel
   int persistent_blocks;  // co-resident CTAs of the persistent form (0: unavailable)
   int use_persistent;     // run the environment phases as one persistent kernel
+  int cluster;            // the persistent form's CTAs are one thread-block cluster
 };
 __host__ __device__ int compact_tiles(int total_slots);
 // Alive list of the current state (ascending slots) and its count.
 cudaError_t launch_compact(const Dev &d, cudaStream_t s);
 // Shared-memory attributes and the persistent form's grid size.
 cudaError_t env_prepare(const Layout &L, EnvGrid *g);
+// A small batch: one cluster of a few CTAs in place of one CTA per SM.
+void env_use_small_grid(const Layout &L, EnvGrid *g);
 cudaError_t launch_env_phases(const Dev &d, const Layout &L, const Rules &R, const EnvGrid &g,
                               cudaStream_t s);
 
