@@ -24,8 +24,9 @@
  *     it, allocates no other device memory, and never frees caller memory.
  *     Each handle holds three small pinned host buffers for the statistics
  *     and status word (about 2 x n_envs x 8 x ECO_N_STATS bytes each; one
- *     for eco_read_stats(), two for eco_step_read()), freed by
- *     eco_destroy(); a read copies into one of them in one transfer.
+ *     for eco_read_stats(), two for eco_step_read()) and, when one of its
+ *     worlds is that small, one of at most 1 MB for eco_read_state(), freed
+ *     by eco_destroy(); a read copies into one of them in one transfer.
  *   - Streams: all device work is enqueued on the stream given to
  *     eco_create() (a cudaStream_t passed as void*; NULL = legacy default
  *     stream).  eco_reset() and eco_step() are asynchronous.  eco_read_*()

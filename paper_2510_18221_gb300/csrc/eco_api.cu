@@ -74,6 +74,8 @@ struct eco_handle {
   size_t rd_bytes;
   int rd_pending;
   cudaEvent_t rd_ev[2];
+  uint8_t *bounce;  // pinned, behind rd_host's slots: a small world's whole state
+  size_t bounce_bytes;
   char err[512];
 };
 
@@ -228,6 +230,12 @@ static Layout make_layout(const eco_config *c) {
 // The parameter staging region holds about this many bytes (one slot at
 // least): transfers of 32 MB run at the host link's rate.
 constexpr long long kStagingBytes = 32ll << 20;
+// Worlds whose whole state fits this are read through pinned memory.
+constexpr size_t kBounceBytes = 1u << 20;
+// Bytes of every array of eco_read_state for N cells and S slots, each padded
+// to 8: 4 plain cell arrays and 6 converted bytes a cell; 7 i32 and 2 u8
+// plain slot arrays and 20 converted bytes a slot; the step.
+static size_t state_bytes(size_t N, size_t S) { return 22 * N + 50 * S + 256; }
 
 // Workspace carving (256-byte aligned regions).
 struct Carve {
@@ -477,6 +485,12 @@ extern "C" int eco_create(const eco_config *cfg, void *dev_workspace, size_t byt
   h->rd_bytes = (size_t)(reinterpret_cast<uint8_t *>(h->d.counters + CNT_N) -
                          reinterpret_cast<uint8_t *>(h->d.stats_total));
   h->rd_host = nullptr;
+  h->bounce = nullptr;
+  h->bounce_bytes = 0;
+  for (int e = 0; e < cfg->n_envs; ++e) {
+    const size_t n = state_bytes((size_t)cfg->env_side[e] * cfg->env_side[e], (size_t)cfg->env_slots[e]);
+    if (n <= kBounceBytes) h->bounce_bytes = std::max(h->bounce_bytes, n);
+  }
   // zero the whole workspace first, then install the environment table
   cudaError_t e = cudaMemsetAsync(h->ws, 0, need, h->stream);
   if (e == cudaSuccess)
@@ -492,7 +506,9 @@ extern "C" int eco_create(const eco_config *cfg, void *dev_workspace, size_t byt
     const long long work = std::max((long long)h->d.total_slots, (long long)h->d.total_cells / 4);
     if (work <= 4096) env_use_small_grid(h->L, &h->grid);
   }
-  if (e == cudaSuccess) e = cudaMallocHost(&h->rd_host, 3 * h->rd_bytes);
+  const size_t rd_all = (3 * h->rd_bytes + 255) & ~(size_t)255;
+  if (e == cudaSuccess) e = cudaMallocHost(&h->rd_host, rd_all + h->bounce_bytes);
+  if (e == cudaSuccess) h->bounce = h->rd_host + rd_all;
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->rd_ev[0], cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->rd_ev[1], cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreate(&h->ev_dummy[0]);
@@ -944,58 +960,96 @@ static int check_env(eco_handle *h, int32_t env) {
   return ECO_OK;
 }
 
+// Write to every page of the caller's output range [p, p + bytes) before the
+// GPU copies into it: pages of a fresh allocation are then faulted in here,
+// in order, by the host (128 MB: 6 ms), instead of by the copy (34 ms).
+static void touch_pages(void *p, size_t bytes) {
+  static const size_t page = (size_t)sysconf(_SC_PAGESIZE);
+  volatile char *c = reinterpret_cast<volatile char *>(p);
+  if (bytes == 0) return;
+  for (size_t at = 0; at < bytes; at += page - ((reinterpret_cast<uintptr_t>(p) + at) & (page - 1))) c[at] = 0;
+}
+
 extern "C" int eco_read_state(eco_handle *h, int32_t env, eco_state_view *out) {
   int rc = check_env(h, env);
   if (rc) return rc;
   if (!out) return fail(h, ECO_EINVAL, "null view");
   const EnvDesc &ed = h->env_host[env];
-  const int N = ed.side * ed.side, S = ed.n_slots;
-  std::vector<uint8_t> cellf(N), alive(S), facing(S);
-  std::vector<int32_t> occ(N), pos(S), energy(S), parent(S), birth(S);
-  long long step = 0;
+  const size_t N = (size_t)ed.side * ed.side, S = (size_t)ed.n_slots;
+  const Dev &d = h->d;
+  const int64_t so = ed.slot_off, co = ed.cell_off;
   cudaStream_t s = h->stream;
-  if (out->hp) CUDA_TRY(h, cudaMemcpyAsync(out->hp, h->d.hp + ed.slot_off, 4 * (size_t)S, cudaMemcpyDeviceToHost, s));
-  if (out->age) CUDA_TRY(h, cudaMemcpyAsync(out->age, h->d.age + ed.slot_off, 4 * (size_t)S, cudaMemcpyDeviceToHost, s));
-  if (out->res) CUDA_TRY(h, cudaMemcpyAsync(out->res, h->d.res + ed.cell_off, 4 * (size_t)N, cudaMemcpyDeviceToHost, s));
-  if (out->water) CUDA_TRY(h, cudaMemcpyAsync(out->water, h->d.water + ed.cell_off, 4 * (size_t)N, cudaMemcpyDeviceToHost, s));
-  if (out->bio) CUDA_TRY(h, cudaMemcpyAsync(out->bio, h->d.bio + ed.cell_off, 4 * (size_t)N, cudaMemcpyDeviceToHost, s));
-  if (out->photo) CUDA_TRY(h, cudaMemcpyAsync(out->photo, h->d.photo + ed.cell_off, 4 * (size_t)N, cudaMemcpyDeviceToHost, s));
-  if (out->a_water) CUDA_TRY(h, cudaMemcpyAsync(out->a_water, h->d.a_water + ed.slot_off, 4 * (size_t)S, cudaMemcpyDeviceToHost, s));
-  if (out->a_bio) CUDA_TRY(h, cudaMemcpyAsync(out->a_bio, h->d.a_bio + ed.slot_off, 4 * (size_t)S, cudaMemcpyDeviceToHost, s));
-  std::vector<float4> colour(out->colour ? S : 0);
-  if (out->colour)
-    CUDA_TRY(h, cudaMemcpyAsync(colour.data(), h->d.colour + ed.slot_off, sizeof(float4) * (size_t)S,
-                                cudaMemcpyDeviceToHost, s));
-  CUDA_TRY(h, cudaMemcpyAsync(cellf.data(), h->d.cellf + ed.cell_off, N, cudaMemcpyDeviceToHost, s));
-  CUDA_TRY(h, cudaMemcpyAsync(occ.data(), h->d.occ + ed.cell_off, 4 * (size_t)N, cudaMemcpyDeviceToHost, s));
-  CUDA_TRY(h, cudaMemcpyAsync(alive.data(), h->d.alive + ed.slot_off, S, cudaMemcpyDeviceToHost, s));
-  CUDA_TRY(h, cudaMemcpyAsync(facing.data(), h->d.facing + ed.slot_off, S, cudaMemcpyDeviceToHost, s));
-  CUDA_TRY(h, cudaMemcpyAsync(pos.data(), h->d.pos + ed.slot_off, 4 * (size_t)S, cudaMemcpyDeviceToHost, s));
-  CUDA_TRY(h, cudaMemcpyAsync(energy.data(), h->d.energy + ed.slot_off, 4 * (size_t)S, cudaMemcpyDeviceToHost, s));
-  CUDA_TRY(h, cudaMemcpyAsync(parent.data(), h->d.parent + ed.slot_off, 4 * (size_t)S, cudaMemcpyDeviceToHost, s));
-  CUDA_TRY(h, cudaMemcpyAsync(birth.data(), h->d.birth + ed.slot_off, 4 * (size_t)S, cudaMemcpyDeviceToHost, s));
-  CUDA_TRY(h, cudaMemcpyAsync(&step, h->d.step, sizeof step, cudaMemcpyDeviceToHost, s));
-  CUDA_TRY(h, cudaStreamSynchronize(s));
-  for (int c = 0; c < N; ++c) {
-    if (out->food) out->food[c] = (cellf[c] & CELL_FOOD) ? 1 : 0;
-    if (out->wall) out->wall[c] = (cellf[c] & CELL_WALL) ? 1 : 0;
-    if (out->occ) out->occ[c] = occ[c] < 0 ? -1 : occ[c] - ed.slot_off;
-  }
-  for (int i = 0; i < S; ++i) {
-    if (out->alive) out->alive[i] = alive[i];
-    if (out->x) out->x[i] = pos[i] % ed.side;
-    if (out->y) out->y[i] = pos[i] / ed.side;
-    if (out->facing) out->facing[i] = facing[i];
-    if (out->energy) out->energy[i] = energy[i];
-    if (out->parent) out->parent[i] = parent[i];
-    if (out->birth_step) out->birth_step[i] = birth[i];
-    if (out->colour) {
-      out->colour[3 * i + 0] = colour[i].x;
-      out->colour[3 * i + 1] = colour[i].y;
-      out->colour[3 * i + 2] = colour[i].z;
+  // arrays the caller gets as the device holds them
+  struct Plain {
+    void *dst;
+    const void *src;
+    size_t bytes;
+  } plain[] = {{out->alive, d.alive + so, S},        {out->facing, d.facing + so, S},
+               {out->energy, d.energy + so, 4 * S},  {out->parent, d.parent + so, 4 * S},
+               {out->birth_step, d.birth + so, 4 * S}, {out->hp, d.hp + so, 4 * S},
+               {out->age, d.age + so, 4 * S},        {out->a_water, d.a_water + so, 4 * S},
+               {out->a_bio, d.a_bio + so, 4 * S},    {out->res, d.res + co, 4 * N},
+               {out->water, d.water + co, 4 * N},    {out->bio, d.bio + co, 4 * N},
+               {out->photo, d.photo + co, 4 * N},    {out->step, d.step, sizeof(int64_t)}};
+  // arrays a kernel converts: every cell's food, wall and env-local occupant
+  // (6 bytes a cell), every slot's x, y and RGB (20 bytes a slot)
+  const size_t staging = (size_t)d.staging_slots * h->L.P * 4;
+  if (state_bytes(N, S) <= std::min(h->bounce_bytes, staging)) {
+    // a small world: everything packed by one kernel and brought over by one
+    // copy into pinned memory (a copy per array cost 0.3 ms)
+    uint8_t *base = reinterpret_cast<uint8_t *>(d.staging);
+    PackList list = {};
+    size_t at = 0;
+    for (const Plain &p : plain) {
+      if (!p.dst) continue;
+      list.src[list.n] = p.src;
+      list.at[list.n] = (uint32_t)at;
+      list.bytes[list.n++] = (uint32_t)p.bytes;
+      at += (p.bytes + 7) & ~(size_t)7;
     }
+    const size_t cells = at, slots = (cells + 6 * N + 7) & ~(size_t)7;
+    CUDA_TRY(h, launch_pack(list, base, s));
+    CUDA_TRY(h, launch_state_out(d, env, 0, (int)N, 0, (int)S, base + cells, base + slots, s));
+    CUDA_TRY(h, cudaMemcpyAsync(h->bounce, base, slots + 20 * S, cudaMemcpyDeviceToHost, s));
+    CUDA_TRY(h, cudaStreamSynchronize(s));
+    const uint8_t *m = h->bounce;
+    int k = 0;
+    for (const Plain &p : plain)
+      if (p.dst) memcpy(p.dst, m + list.at[k++], p.bytes);
+    if (out->occ) memcpy(out->occ, m + cells, 4 * N);
+    if (out->food) memcpy(out->food, m + cells + 4 * N, N);
+    if (out->wall) memcpy(out->wall, m + cells + 5 * N, N);
+    if (out->x) memcpy(out->x, m + slots, 4 * S);
+    if (out->y) memcpy(out->y, m + slots + 4 * S, 4 * S);
+    if (out->colour) memcpy(out->colour, m + slots + 8 * S, 12 * S);
+    return ECO_OK;
   }
-  if (out->step) *out->step = step;
+  auto copy = [&](void *dst, const void *src, size_t bytes) -> cudaError_t {
+    if (!dst || !bytes) return cudaSuccess;
+    touch_pages(dst, bytes);
+    return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, s);
+  };
+  // converted arrays in pieces of the staging region, a multiple of 4 cells
+  uint8_t *base = reinterpret_cast<uint8_t *>(d.staging);
+  const size_t cell_piece = std::max<size_t>(4, staging / 6 / 4 * 4), slot_piece = std::max<size_t>(1, staging / 20);
+  if (out->food || out->wall || out->occ)
+    for (size_t c = 0; c < N; c += cell_piece) {
+      const size_t n = std::min(cell_piece, N - c);
+      CUDA_TRY(h, launch_state_out(d, env, (int)c, (int)n, 0, 0, base, base, s));
+      CUDA_TRY(h, copy(out->occ ? out->occ + c : nullptr, base, 4 * n));
+      CUDA_TRY(h, copy(out->food ? out->food + c : nullptr, base + 4 * n, n));
+      CUDA_TRY(h, copy(out->wall ? out->wall + c : nullptr, base + 5 * n, n));
+    }
+  if (out->x || out->y || out->colour)
+    for (size_t i = 0; i < S; i += slot_piece) {
+      const size_t n = std::min(slot_piece, S - i);
+      CUDA_TRY(h, launch_state_out(d, env, 0, 0, (int)i, (int)n, base, base, s));
+      CUDA_TRY(h, copy(out->x ? out->x + i : nullptr, base, 4 * n));
+      CUDA_TRY(h, copy(out->y ? out->y + i : nullptr, base + 4 * n, 4 * n));
+      CUDA_TRY(h, copy(out->colour ? out->colour + 3 * i : nullptr, base + 8 * n, 12 * n));
+    }
+  for (const Plain &p : plain) CUDA_TRY(h, copy(p.dst, p.src, p.bytes));
+  CUDA_TRY(h, cudaStreamSynchronize(s));
   return ECO_OK;
 }
 
@@ -1133,16 +1187,6 @@ static int check_range(eco_handle *h, int32_t env, int32_t slot0, int32_t n) {
   if (rc) return rc;
   if (slot0 < 0 || n < 0 || slot0 + n > h->env_host[env].n_slots) return fail(h, ECO_EINVAL, "slot range out of bounds");
   return ECO_OK;
-}
-
-// Write to every page of the caller's output range [p, p + bytes) before the
-// GPU copies into it: pages of a fresh allocation are then faulted in here,
-// in order, by the host (128 MB: 6 ms), instead of by the copy (34 ms).
-static void touch_pages(void *p, size_t bytes) {
-  static const size_t page = (size_t)sysconf(_SC_PAGESIZE);
-  volatile char *c = reinterpret_cast<volatile char *>(p);
-  if (bytes == 0) return;
-  for (size_t at = 0; at < bytes; at += page - ((reinterpret_cast<uintptr_t>(p) + at) & (page - 1))) c[at] = 0;
 }
 
 extern "C" int eco_read_params(eco_handle *h, int32_t env, int32_t slot0, int32_t n, float *out) {

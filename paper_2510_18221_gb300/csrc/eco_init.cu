@@ -1,6 +1,7 @@
 // eco_init.cu -- reset of every environment (Sec. 3.2: grid world with
-// randomly distributed resources and a founding population) and the recount
-// of the statistics after a state write.  The founders' weights are drawn in
+// randomly distributed resources and a founding population), the recount
+// of the statistics after a state write, and the state in the form its
+// readers get.  The founders' weights are drawn in
 // eco_params.cu.
 //
 // Founders: the K non-wall cells with the smallest 64-bit keys
@@ -436,6 +437,65 @@ __global__ void __launch_bounds__(1024) k_recount(Dev d, Rules R) {
     tot[ST_BIO_AGENTS] = last[ST_BIO_AGENTS] = terrain ? bat : 0;
     tot[ST_STEP] = last[ST_STEP] = t;
   }
+}
+
+__global__ void __launch_bounds__(256) k_pack(PackList list, uint8_t *base) {
+  const int k = blockIdx.y;
+  const uint8_t *src = reinterpret_cast<const uint8_t *>(list.src[k]);
+  uint8_t *dst = base + list.at[k];
+  const uint32_t n = list.bytes[k], i0 = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+  // slot arrays of bytes may start at any address; words where they allow it
+  if ((((uintptr_t)src | n) & 3u) == 0u)
+    for (uint32_t i = i0; i < n / 4; i += step)
+      reinterpret_cast<uint32_t *>(dst)[i] = reinterpret_cast<const uint32_t *>(src)[i];
+  else
+    for (uint32_t i = i0; i < n; i += step) dst[i] = src[i];
+}
+
+cudaError_t launch_pack(const PackList &list, uint8_t *base, cudaStream_t s) {
+  if (list.n == 0) return cudaSuccess;
+  k_pack<<<dim3(8, list.n), 256, 0, s>>>(list, base);
+  return cudaGetLastError();
+}
+
+__global__ void __launch_bounds__(256) k_state_out(Dev d, int env, int c0, int nc, int s0, int ns, uint8_t *cells,
+                                                   uint8_t *slots) {
+  const EnvDesc ed = d.env[env];
+  const int g0 = blockIdx.x * blockDim.x + threadIdx.x, gs = gridDim.x * blockDim.x;
+  int32_t *occ = reinterpret_cast<int32_t *>(cells);
+  uint8_t *food = cells + 4 * (size_t)nc, *wall = cells + 5 * (size_t)nc;
+  for (int g = g0; g < nc / 4; g += gs) {  // sides are even: whole groups of four
+    const int c = ed.cell_off + c0 + 4 * g;
+    const uchar4 cf = *reinterpret_cast<const uchar4 *>(d.cellf + c);
+    int4 o = *reinterpret_cast<const int4 *>(d.occ + c);
+    o.x = o.x < 0 ? -1 : o.x - ed.slot_off;
+    o.y = o.y < 0 ? -1 : o.y - ed.slot_off;
+    o.z = o.z < 0 ? -1 : o.z - ed.slot_off;
+    o.w = o.w < 0 ? -1 : o.w - ed.slot_off;
+    occ[4 * g] = o.x, occ[4 * g + 1] = o.y, occ[4 * g + 2] = o.z, occ[4 * g + 3] = o.w;
+    const uint8_t v[4] = {cf.x, cf.y, cf.z, cf.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      food[4 * g + k] = (v[k] & CELL_FOOD) ? 1 : 0;
+      wall[4 * g + k] = (v[k] & CELL_WALL) ? 1 : 0;
+    }
+  }
+  int32_t *x = reinterpret_cast<int32_t *>(slots), *y = x + ns;
+  float *rgb = reinterpret_cast<float *>(y + ns);
+  for (int i = g0; i < ns; i += gs) {
+    const int s = ed.slot_off + s0 + i, p = d.pos[s];
+    x[i] = p % ed.side;
+    y[i] = p / ed.side;
+    const float4 c = d.colour[s];
+    rgb[3 * i] = c.x, rgb[3 * i + 1] = c.y, rgb[3 * i + 2] = c.z;
+  }
+}
+
+cudaError_t launch_state_out(const Dev &d, int env, int c0, int nc, int s0, int ns, uint8_t *cells, uint8_t *slots,
+                             cudaStream_t s) {
+  const int work = nc / 4 > ns ? nc / 4 : ns;
+  k_state_out<<<grid_for(work, 256, 1024), 256, 0, s>>>(d, env, c0, nc, s0, ns, cells, slots);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_init_static(const Dev &d, const EnvGrid &g, cudaStream_t s) {

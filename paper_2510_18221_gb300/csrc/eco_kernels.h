@@ -66,6 +66,21 @@ cudaError_t launch_reset(const Dev &d, const Layout &L, const Rules &R, const En
 cudaError_t launch_init_static(const Dev &d, const EnvGrid &g, cudaStream_t s);
 // Recompute the "now" statistics (alive, food, energy, step) from the state.
 cudaError_t launch_recount(const Dev &d, const Rules &R, cudaStream_t s);
+// State I/O (eco_init.cu).  Pieces of device memory, packed one behind the
+// other at `base`.
+constexpr int kPackMost = 16;
+struct PackList {
+  int n;
+  const void *src[kPackMost];
+  uint32_t at[kPackMost], bytes[kPackMost];  // at: a multiple of 8
+};
+cudaError_t launch_pack(const PackList &list, uint8_t *base, cudaStream_t s);
+// Cells [c0, c0 + nc) (c0 a multiple of 4) of environment env to `cells`: the
+// env-local occupants (i32), then food, then wall (u8); slots [s0, s0 + ns) to
+// `slots`: x, then y (i32), then RGB (3 f32).
+cudaError_t launch_state_out(const Dev &d, int env, int c0, int nc, int s0, int ns, uint8_t *cells, uint8_t *slots,
+                             cudaStream_t s);
+
 // Placement tiles of a world of side L (reset).
 int place_tiles(int side);
 
