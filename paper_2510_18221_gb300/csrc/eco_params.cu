@@ -25,14 +25,14 @@ namespace {
 constexpr int kParThreads = 512;
 constexpr int kMaxRows = 32;
 
-// Row stride of a tile of rows of nin inputs.  Rows whose length is a
-// multiple of 4 are padded to an odd number of 16-byte units, so that 32
-// lanes reading the same unit of their own rows as float4 hit every bank
-// once per quarter-warp.  Other rows (every D of 3 k^2 + 4 or 8 is odd) stay
-// packed, in logical order with the first Philox block's offset, and are
-// read element by element, one bank per lane when nin is odd.
+// Row stride of a tile of rows of nin inputs.  The tile is read four rows per
+// lane, eight lanes to an input (32-row tiles), so rows four apart should
+// differ by an odd multiple of 4 banks: rows of an odd length (every D of
+// 3 k^2 + 4 or 8) stay packed, in logical order with the first Philox block's
+// offset.  Rows of a multiple of 4 are padded by 2, an odd multiple of 8
+// banks (two lanes per bank), and still take a block's normals as pairs.
 __host__ __device__ inline bool tile_by4(int nin) { return (nin & 3) == 0; }
-__host__ __device__ inline int tile_stride(int nin) { return tile_by4(nin) && ((nin >> 2) & 1) == 0 ? nin + 4 : nin; }
+__host__ __device__ inline int tile_stride(int nin) { return tile_by4(nin) ? nin + 2 : nin; }
 
 size_t tile_bytes(const Layout &L, int rows) {
   // k_params_in's row strides and k_params_out's
@@ -63,6 +63,45 @@ __device__ __forceinline__ float fp8_scale(float mx) {
   return s == 0.0f ? 1.0f : s;
 }
 
+// Philox4x32-10 of counter (c0, c1, 0, 0) under round keys made once (the
+// same key serves a whole agent; the key schedule was a quarter of the
+// generator's instructions).
+struct PhiloxKeys {
+  uint32_t k0[10], k1[10];
+  __device__ __forceinline__ PhiloxKeys(uint32_t a, uint32_t b) {
+#pragma unroll
+    for (int i = 0; i < 10; ++i) {
+      k0[i] = a + (uint32_t)i * 0x9E3779B9u;
+      k1[i] = b + (uint32_t)i * 0xBB67AE85u;
+    }
+  }
+  __device__ __forceinline__ U4 draw(uint32_t c0, uint32_t c1) const {
+    uint32_t c2 = 0u, c3 = 0u;
+#pragma unroll
+    for (int i = 0; i < 10; ++i) {
+      const uint32_t a0 = 0xD2511F53u * c0, h0 = __umulhi(0xD2511F53u, c0);
+      const uint32_t a2 = 0xCD9E8D57u * c2, h2 = __umulhi(0xCD9E8D57u, c2);
+      c0 = h2 ^ c1 ^ k0[i];
+      c1 = a2;
+      c2 = h0 ^ c3 ^ k1[i];
+      c3 = a0;
+    }
+    return U4{c0, c1, c2, c3};
+  }
+};
+
+// n / f correctly rounded, f = sqrt(fan-in) with its correctly rounded
+// reciprocal r: one correction of the quotient n r (Markstein, "Computation
+// of elementary functions on the IBM RISC System/6000 processor", 1990;
+// Brisebarre, Muller and Raina, IEEE TC 53(8), 2004, on divisors known in
+// advance).  Equal to the IEEE quotient for every significand of n and every
+// fan-in the configuration allows, checked exhaustively; n is 0 or of normal
+// magnitude, so no scaling is needed.
+__device__ __forceinline__ float divide_by_known(float n, float f, float r) {
+  const float q = n * r;
+  return fmaf(fmaf(-q, f, n), r, q);
+}
+
 }  // namespace
 
 // Parameters of slots [slot0, slot0 + n) into their blocks, with the streamed
@@ -75,11 +114,13 @@ __device__ __forceinline__ float fp8_scale(float mx) {
 // all zero, with FP8 scales of 1.
 // Bound by the arithmetic of the normals beside the writes: 65,536 slots of
 // 371-64-64-9 BF16 are 11.2 GB, 1.7 ms at the copy rate, and the whole reset
-// takes 4.6 ms (19.4 ms with a Philox block per element, the streamed copy
+// takes 3.8 ms (19.4 ms with a Philox block per element, the streamed copy
 // from a second pass over the masters and one CTA per world placing the
-// founders); 683-128-128-9 FP8, 41.5 GB, 19 ms (231 ms, mostly FP8 rows read
-// with a stride).  512 threads at 64 registers: 256 or 512 threads with 2 to
-// 6 CTAs per SM lie within 5% in BF16, and up to 30% above in FP8.
+// founders; 4.6 ms with the key schedule in every block, an IEEE division per
+// weight and one row per lane); 683-128-128-9 FP8, 41.5 GB, 16.6 ms (231 ms,
+// mostly FP8 rows read with a stride; 19 ms).  512 threads at 64 registers:
+// 256 or 512 threads with 2 to 6 CTAs per SM lie within 5% in BF16, and up to
+// 30% above in FP8.
 //
 // Otherwise: from `flat`, [n][P] in logical order, the caller's parameters
 // on the device.
@@ -92,14 +133,15 @@ __global__ void __launch_bounds__(kParThreads, 2)
   const int D = L.D, H = L.H, A = L.A;
   const int tid = threadIdx.x, nt = kParThreads, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
   const int64_t mper = L.mstride / 4;
-  // the scale of each fan-in (layout_fan_in), once per CTA: a factor in the
-  // paper form, a divisor in the plain form
+  // the scale of each fan-in (layout_fan_in), once per CTA: in the paper form
+  // a factor, in the plain form (two fan-ins, D and H) a divisor
   auto scale_of = [&](int q) {
     const float fan = (float)layout_fan_in(L, q);
     return L.relu ? sqrtf(__fdiv_rn(2.0f, fan)) : sqrtf(fan);
   };
   const float f_vision = scale_of(0), f_internal = scale_of(L.patch * H), f_compass = scale_of((L.patch + 1) * H);
   const float f_hidden = scale_of(D * H);
+  const float r_in = __frcp_rn(f_vision), r_hidden = __frcp_rn(f_hidden);
   for (int i = blockIdx.x; i < n; i += gridDim.x) {
     const int s = slot0 + i;
     const float *in = INIT ? nullptr : flat + (int64_t)i * L.P;
@@ -130,15 +172,18 @@ __global__ void __launch_bounds__(kParThreads, 2)
         const int shift = INIT && !by4 ? lbase & 3 : 0;  // rows of a multiple of 4 start a block
         if (INIT) {
           const int b0 = lbase >> 2, b1 = (lbase + nel - 1) >> 2;
+          const PhiloxKeys keys(ed.seed, S_W_INIT);
           for (int g = b0 + tid; g <= b1; g += nt) {
             float n4[4];
-            normals4(philox(ls, (uint32_t)g, 0u, 0u, ed.seed, S_W_INIT), n4);
+            normals4(keys.draw(ls, (uint32_t)g), n4);
             int at = 4 * (g - b0);
             if (by4) {
-              const int rr = at / nin;
-              at += rr * (rs - nin);
+              at += (at / nin) * (rs - nin);
+              *reinterpret_cast<float2 *>(tile + at) = make_float2(n4[0], n4[1]);
+              *reinterpret_cast<float2 *>(tile + at + 2) = make_float2(n4[2], n4[3]);
+            } else {
+              *reinterpret_cast<float4 *>(tile + at) = make_float4(n4[0], n4[1], n4[2], n4[3]);
             }
-            *reinterpret_cast<float4 *>(tile + at) = make_float4(n4[0], n4[1], n4[2], n4[3]);
           }
         } else {
           for (int rr = warp; rr < R; rr += nw)
@@ -146,41 +191,46 @@ __global__ void __launch_bounds__(kParThreads, 2)
         }
         if (PREC == PREC_FP8 && tid < R) s_max[tid] = 0u;
         __syncthreads();
-        // 2. (INIT: scaled) to the master and the BF16 copy: lane = row
-        const int rr = lane & (R - 1), sub = lane >> rlog, per = 32 >> rlog;
-        float *row = tile + shift + rr * rs;
-        float mx = 0.0f;
-        auto put = [&](int j, float n) -> float {
-          const int q = qbase + j * H + o0 + rr;
-          float v = n;
+        // 2. (INIT: scaled) to the master and the BF16 copy: a lane takes four
+        // rows of one input
+        const int wlog = rlog - 2, wd = lane & ((1 << wlog) - 1), per = 32 >> wlog;
+        float *row = tile + shift + 4 * wd * rs;
+        float mx[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        for (int j = warp * per + (lane >> wlog); j < nin; j += nw * per) {
+          float v[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) v[k] = row[k * rs + j];
           if (INIT) {
-            const float f = layer > 0 ? f_hidden : j < L.patch ? f_vision
-                            : (j > L.patch && j < L.patch + 5) ? f_compass : f_internal;
-            v = L.relu ? n * f : __fdiv_rn(n, f);
+            if (L.relu) {
+              const float f = layer > 0 ? f_hidden : j < L.patch ? f_vision
+                              : (j > L.patch && j < L.patch + 5) ? f_compass : f_internal;
+#pragma unroll
+              for (int k = 0; k < 4; ++k) v[k] *= f;
+            } else {
+              const float f = layer > 0 ? f_hidden : f_vision, r = layer > 0 ? r_hidden : r_in;
+#pragma unroll
+              for (int k = 0; k < 4; ++k) v[k] = divide_by_known(v[k], f, r);
+            }
           }
-          m[q] = v;
-          if (PREC == PREC_BF16) reinterpret_cast<__nv_bfloat16 *>(blk)[q] = __float2bfloat16_rn(v);
-          if (PREC == PREC_FP8) mx = fmaxf(mx, fabsf(v));
-          return v;
-        };
-        if (by4) {
-          for (int c = warp * per + sub; c < (nin >> 2); c += nw * per) {
-            float4 v = *reinterpret_cast<const float4 *>(row + 4 * c);
-            v.x = put(4 * c, v.x);
-            v.y = put(4 * c + 1, v.y);
-            v.z = put(4 * c + 2, v.z);
-            v.w = put(4 * c + 3, v.w);
-            if (INIT && PREC == PREC_FP8) *reinterpret_cast<float4 *>(row + 4 * c) = v;
+          const int q = qbase + j * H + o0 + 4 * wd;
+          *reinterpret_cast<float4 *>(m + q) = make_float4(v[0], v[1], v[2], v[3]);
+          if (PREC == PREC_BF16) {
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(v[0], v[1]), hi = __floats2bfloat162_rn(v[2], v[3]);
+            *reinterpret_cast<uint2 *>(reinterpret_cast<__nv_bfloat16 *>(blk) + q) =
+                make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
           }
-        } else {
-          for (int j = warp * per + sub; j < nin; j += nw * per) {
-            const float v = put(j, row[j]);
-            if (INIT && PREC == PREC_FP8) row[j] = v;
+          if (PREC == PREC_FP8) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              if (INIT) row[k * rs + j] = v[k];
+              mx[k] = fmaxf(mx[k], fabsf(v[k]));
+            }
           }
         }
         if (PREC == PREC_FP8) {
           // non-negative floats compare as their bits
-          atomicMax(&s_max[rr], __float_as_uint(mx));
+#pragma unroll
+          for (int k = 0; k < 4; ++k) atomicMax(&s_max[4 * wd + k], __float_as_uint(mx[k]));
           __syncthreads();
           if (tid < R) {
             const float sc = fp8_scale(__uint_as_float(s_max[tid]));
