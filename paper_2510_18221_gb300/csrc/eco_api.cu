@@ -328,10 +328,11 @@ static size_t carve(const eco_config *c, const Layout &L, uint8_t *base, Dev *d,
   D.trace = k.take<unsigned long long>((size_t)kTraceSteps * kTraceWords);
   D.staging_slots = (int)std::min(slots, std::max(1ll, kStagingBytes / (4ll * L.P)));
   D.staging = k.take<float>((size_t)D.staging_slots * L.P);
-  // The policy kernel's FP8 tail batches load up to kStreamSlack bytes past
-  // the last weight block (their products are skipped): the regions after
-  // the weights (the histogram alone is 256 KB per world) keep those loads
-  // inside the workspace, and this keeps that true for any layout.
+  // The policy kernel's FP8 tail batches and its requests into L1 reach up
+  // to kStreamSlack bytes past the last weight block (no product uses them):
+  // the regions after the weights (the histogram alone is 256 KB per world)
+  // keep those loads inside the workspace, and this keeps that true for any
+  // layout.
   if (k.off < wq_end + kStreamSlack) k.take<uint8_t>(wq_end + kStreamSlack - k.off);
   return (k.off + 255) & ~(size_t)255;
 }

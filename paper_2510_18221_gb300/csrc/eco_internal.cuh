@@ -338,8 +338,9 @@ __device__ __forceinline__ T *mirror_of(const Dev &d, const T *p) {
 constexpr int kAliveRing = 4096;
 // Readable workspace bytes after the last slot's weight block: the policy
 // kernel's last, partial FP8 batch of a layer loads up to 32 lanes x 8 units
-// x 16 B past the layer's end (and skips those products).
-constexpr int kStreamSlack = 4096;
+// x 16 B past the layer's end (and skips those products), and its requests
+// into L1 run up to four such batches past it.
+constexpr int kStreamSlack = 16384;
 
 // Words of Dev::barrier: the persistent form's grid-barrier arrival counts
 // (one per step parity: a launch uses its step's word and clears the other

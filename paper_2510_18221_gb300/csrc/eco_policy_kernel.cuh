@@ -44,6 +44,21 @@ __device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
+// Request the 128-byte line of p into L1.
+__device__ __forceinline__ void prefetch_l1(const void *p) {
+  asm volatile("prefetch.global.L1 [%0];" ::"l"(p) : "memory");
+}
+
+// Batches that a warp's weight stream is requested into L1 ahead of its loads
+// when few agents are alive (k_policy).
+constexpr int kAheadBatches = 3;
+
+// Lines of the batch of 32 * UNROLL units at p, one per lane.
+template <int UNROLL>
+__device__ __forceinline__ void prefetch_batch(const uint4 *p, int lane) {
+  if (lane < 4 * UNROLL) prefetch_l1(p + 8 * lane);
+}
+
 __device__ __forceinline__ uint4 ldg_stream(const uint4 *p) {
   uint4 r;
   asm("ld.global.nc.L1::no_allocate.L2::256B.v4.u32 {%0,%1,%2,%3}, [%4];"
@@ -246,7 +261,9 @@ __device__ __forceinline__ void layer_finish(float *acc, const float *__restrict
 // nonzero entries of x): a row is the H outputs of one input, UPJ whole
 // units, so the loads stay 16-byte and contiguous per row.  Skipped inputs
 // are exact zeros, whose products add nothing.
-template <int PREC, int H, int UNROLL, bool SPARSE>
+// AHEAD: every batch requests the one kAheadBatches later into L1 (past the
+// layer's end too: the next section, or other regions of the workspace).
+template <int PREC, int H, int UNROLL, bool SPARSE, bool AHEAD>
 __device__ __forceinline__ void layer_in_major(const uint4 *__restrict__ w, int n_in,
                                                const float *__restrict__ x,
                                                const float *__restrict__ bias, int nbias,
@@ -257,7 +274,7 @@ __device__ __forceinline__ void layer_in_major(const uint4 *__restrict__ w, int 
   constexpr int UPJ = H / E;  // units per input
   constexpr int LG = Log2<UPJ>::v;
   static_assert((1 << LG) == UPJ && UPJ <= 32, "H / E must be a power of two <= 32");
-  static_assert(32 * UNROLL * 16 <= kStreamSlack, "a tail batch reads past the layer's end");
+  static_assert((kAheadBatches + 1) * 32 * UNROLL * 16 <= kStreamSlack, "a tail batch reads past the layer's end");
   float acc[E];
 #pragma unroll
   for (int e = 0; e < E; ++e) acc[e] = 0.0f;
@@ -269,6 +286,7 @@ __device__ __forceinline__ void layer_in_major(const uint4 *__restrict__ w, int 
     const int U1 = min(U, (n_exact * UPJ) / (32 * UNROLL) * (32 * UNROLL));
     for (; u < U1; u += 32 * UNROLL) {
       uint4 v[UNROLL];
+      if constexpr (AHEAD) prefetch_batch<UNROLL>(w + (u - lane) + 32 * UNROLL * kAheadBatches, lane);
 #pragma unroll
       for (int k = 0; k < UNROLL; ++k) v[k] = ldg_stream(w + u + 32 * k);
 #pragma unroll
@@ -279,6 +297,7 @@ __device__ __forceinline__ void layer_in_major(const uint4 *__restrict__ w, int 
   for (; u + 32 * (UNROLL - 1) < U; u += 32 * UNROLL) {
     uint4 v[UNROLL];
     int j[UNROLL];
+    if constexpr (AHEAD) prefetch_batch<UNROLL>(w + (u - lane) + 32 * UNROLL * kAheadBatches, lane);
 #pragma unroll
     for (int k = 0; k < UNROLL; ++k) {
       const int uu = u + 32 * k;
@@ -727,7 +746,19 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
   const int G = gridDim.x * WARPS;
   const int rounds = (n_alive + G - 1) / G;
   const int G_eff = (PREC != PREC_FP8 && rounds > 0) ? (n_alive + rounds - 1) / rounds : G;
-  const int w0 = blockIdx.x * WARPS + warp;
+  // Few agents (at most 3/8 of the resident warps): a warp's stream is bound
+  // by the latency of its own batches, so the lines of W_in's next three are
+  // requested into L1 (12 KB a warp; twelve warps' lines fit beside their
+  // observations), the first ones before the observation is gathered, and
+  // the agents are spread over the CTAs.  Variant 6, us on GB300, 600 and 1,200
+  // agents with their weights in L2: 371-64-64-9 BF16 22.9 -> 17.2 and 24.9 ->
+  // 18.9, FP32 33.1 -> 25.2 and 35.2 -> 29.4, FP8 15.2 -> 12.8 and 17.0 -> 14.9;
+  // 500-64-64-64-9 BF16 35.5 -> 27.1 and 37.2 -> 29.0 (from HBM 43.6 -> 37.5 and
+  // 45.7 -> 39.6).  Where the line lies: 2,400 agents gain from L2 (29.0 -> 23.2)
+  // and lose from HBM (35.5 -> 39.6), 4,800 lose in both (45.5 -> 49.3), their
+  // stream being bound by bandwidth.
+  const bool few = 8 * n_alive <= 3 * G;
+  const int w0 = few ? warp * (int)gridDim.x + (int)blockIdx.x : (int)blockIdx.x * WARPS + warp;
   // At the start of the launch every warp gathers an observation with no
   // weights in flight: the first 4 KB of each warp's first agent's weights
   // are requested into L2 before that gather.
@@ -751,6 +782,11 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
     const int slot = slot_n, env = env_n, pos = pos_n, f = f_n;
     const bool more = i + G_eff < n_alive;
     if (more) slot_n = d.alive_list[i + G_eff];
+    if (!SPARSE && few) {
+#pragma unroll
+      for (int q = 0; q < kAheadBatches; ++q)
+        prefetch_batch<UNROLL>(reinterpret_cast<const uint4 *>(d.wq + (int64_t)slot * L.stride) + 32 * UNROLL * q, lane);
+    }
     if (env != e_cur) {
       flush();
       e_cur = env;
@@ -781,21 +817,25 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
 
     // -- input layer: act(sum over sensors of (W_s x_s + b_s)) -> hs
     if constexpr (SPARSE) {
-      layer_in_major<PREC, H, UNROLL, true>(wb + L.off_w1 / 16, n_nz, xs, bias, L.ns, scale, hs,
-                                            lane, L.relu, idx);
+      layer_in_major<PREC, H, UNROLL, true, false>(wb + L.off_w1 / 16, n_nz, xs, bias, L.ns, scale, hs,
+                                                   lane, L.relu, idx);
     } else {
       // one-hot vision: the patch inputs are 0 or 1, exact in f16
-      layer_in_major<PREC, H, UNROLL, false>(wb + L.off_w1 / 16, L.D, xs, bias, L.ns, scale, hs,
-                                             lane, L.relu, nullptr,
-                                             R.vision == VISION_CHANNELS ? L.patch : 0);
+      const int n_exact = R.vision == VISION_CHANNELS ? L.patch : 0;
+      if (few)
+        layer_in_major<PREC, H, UNROLL, false, true>(wb + L.off_w1 / 16, L.D, xs, bias, L.ns, scale, hs, lane,
+                                                     L.relu, nullptr, n_exact);
+      else
+        layer_in_major<PREC, H, UNROLL, false, false>(wb + L.off_w1 / 16, L.D, xs, bias, L.ns, scale, hs, lane,
+                                                      L.relu, nullptr, n_exact);
     }
     __syncwarp();
     // -- hidden layers: h = act(W_l h + b_l), alternating between hs and xs
     float *cur = hs, *nxt = xs;
     for (int l = 0; l < L.L; ++l) {
-      layer_in_major<PREC, H, UNROLL, false>(wb + (L.off_w2 + l * H * H * L.es) / 16, H, cur,
-                                             bias + L.ns * H + l * H, 1, scale + H + l * H, nxt,
-                                             lane, L.relu, nullptr);
+      layer_in_major<PREC, H, UNROLL, false, false>(wb + (L.off_w2 + l * H * H * L.es) / 16, H, cur,
+                                                    bias + L.ns * H + l * H, 1, scale + H + l * H, nxt,
+                                                    lane, L.relu, nullptr);
       __syncwarp();
       float *tmp = cur;
       cur = nxt;
@@ -1059,8 +1099,8 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
     const float *bias = reinterpret_cast<const float *>(blk + L.off_bias);
     const float *scale = reinterpret_cast<const float *>(blk + L.off_scale);
     if constexpr (SPARSE) {
-      layer_in_major<PREC, H, 8, true>(reinterpret_cast<const uint4 *>(blk), n_nz, xs, bias, L.ns, scale, hs, lane,
-                                       L.relu, idx);
+      layer_in_major<PREC, H, 8, true, false>(reinterpret_cast<const uint4 *>(blk), n_nz, xs, bias, L.ns, scale, hs,
+                                              lane, L.relu, idx);
     } else {
       // one-hot vision: the patch inputs are 0 or 1, exact in f16
       ring_layer<PREC, H, NB, UB, SPARSE>(ring, L, L.D, xs, bias, L.ns, scale, hs, lane,
