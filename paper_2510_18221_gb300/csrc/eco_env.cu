@@ -790,14 +790,18 @@ __device__ void ph_birth_assign(const Dev &d, const Rules &R, int b0, int bs, Bi
 // slot, p / 4) for logical parameter p; then the child's streamed BF16 /
 // FP8 copy is re-derived from its new master.
 //
-// Work items per birth: H/8 tiles of W_in (8 output rows x all D inputs),
-// H/8 tiles of each hidden layer, and one item for W_out and the biases
-// (small tiles: a step's few births spread over many CTAs).  A tile draws its
-// normals in logical order (one Philox block per four parameters) into
-// shared memory, then walks the master in its physical (input-major) order
-// so global reads and writes are contiguous; FP8 row scales come from the
-// tile's complete rows.  Block-level (any multiple of 32 threads).
-// ---------------------------------------------------------------------------
+// Work items per birth: tiles of W_in (8 output rows x all D inputs, or fewer
+// rows while a few births leave CTAs idle), of each hidden layer, and one
+// item for W_out and the biases.  A tile's threads request the parent's
+// elements, draw its normals in logical order (one Philox block per four
+// parameters) into shared memory, then write the master in its physical
+// (input-major) order, so global reads and writes are contiguous; a thread
+// keeps its elements, all of one row, for the FP8 codes, whose row scales come
+// from the tile's complete rows.  Block-level (any multiple of 32 threads).
+// 371-64-64-9 FP8, us from the last barrier to the step's end, medians, against
+// tiles always of 8 rows that went through shared memory three times: 4 to 9
+// claimants (3,400 agents) 9.8 -> 7.9, 20 to 39 (12,000) 20.8 -> 18.0; 1 to 3
+// among 12,000 agents, bound by cold code and masters, 12.0 as before.
 constexpr int kMutRows = 8;
 constexpr int kMutRowsLog2 = 3;
 static_assert((1 << kMutRowsLog2) == kMutRows, "kMutRows is a power of two");
@@ -809,10 +813,14 @@ __device__ __forceinline__ uint8_t e4m3_sat(float v) {
 // The births are (par[b], chi[b]) for b < nbirths when par is given (the
 // fast path's pairs in shared memory), else the births list.
 __device__ void ph_mutate(const Dev &d, const Layout &L, const Rules &R, int b0, int bs, float *msm,
-                          float *s_scale, uint32_t t, const int *par, const int *chi, int nbirths) {
+                          uint32_t *s_max, uint32_t t, const int *par, const int *chi, int nbirths) {
   const int D = L.D, H = L.H, A = L.A;
   const int nb = par ? nbirths : d.counters[CNT_N_BIRTHS];
-  const int tiles = H / kMutRows;
+  // rows of a tile: 8, or 4 or 2 while a few births' tiles still find a CTA
+  // each (one SM's arithmetic is a tile's cost: 1 us for 8 rows of 371)
+  int rlog = 1;
+  while (rlog < kMutRowsLog2 && nb * ((((1 + L.L) * H) >> rlog) + 1) > bs) ++rlog;
+  const int rows = 1 << rlog, tiles = H >> rlog;
   const int wtiles = (1 + L.L) * tiles;  // W_in, then each hidden layer
   const int items = wtiles + 1;
   const int tid = threadIdx.x, nt = blockDim.x;
@@ -828,16 +836,28 @@ __device__ void ph_mutate(const Dev &d, const Layout &L, const Rules &R, int b0,
     float *cm = d.master + (int64_t)pc.y * mper;
     uint8_t *cq = d.wq + (int64_t)pc.y * L.stride;
     if (it < wtiles) {
+      constexpr int kHeld = 4;  // elements a thread keeps: tiles of up to 4 nt
       const int layer = it / tiles;  // 0: W_in; l + 1: hidden layer l
       const bool l1 = layer == 0;
-      const int o0 = (it - layer * tiles) * kMutRows;
+      const int o0 = (it - layer * tiles) * rows;
       const int nin = l1 ? D : H;
       const int rs = nin + 1;  // padded shared-memory row stride
       // logical (o0, 0) and the physical start of the layer
       const int lbase = l1 ? o0 * D : D * H + L.ns * H + (layer - 1) * (H * H + H) + o0 * H;
       const int qbase = l1 ? 0 : D * H + (layer - 1) * H * H;
       const int srow = l1 ? 0 : H + (layer - 1) * H;  // first FP8 scale row of the layer
-      const int nel = kMutRows * nin;
+      const int nel = rows * nin;
+      // the parent's master is read-only in this launch (parents and
+      // children are different slots): its elements, this thread's all of
+      // one output row, are requested before the normals are drawn
+      const int rr0 = tid & (rows - 1), q0 = qbase + o0 + rr0;
+      float v[kHeld];
+#pragma unroll
+      for (int k = 0; k < kHeld; ++k) {
+        const int idx = tid + k * nt;
+        v[k] = idx < nel ? __ldg(pm + q0 + (idx >> rlog) * H) : 0.0f;
+      }
+      if (R.precision == PREC_FP8 && tid < kMutRows) s_max[tid] = 0u;
       const int g0 = lbase >> 2, g1 = (lbase + nel - 1) >> 2;
       for (int g = g0 + tid; g <= g1; g += nt) {
         const U4 r = philox(t, lp, (uint32_t)g, 0u, ed.seed, S_MUTATE);
@@ -858,41 +878,50 @@ __device__ void ph_mutate(const Dev &d, const Layout &L, const Rules &R, int b0,
         }
       }
       __syncthreads();
-      // the parent's master is read-only in this launch (parents and
-      // children are different slots), so its loads need not wait for the
-      // child's stores
-#pragma unroll 4
-      for (int idx = tid; idx < nel; idx += nt) {
-        const int j = idx >> kMutRowsLog2, rr = idx & (kMutRows - 1);
-        const int q = qbase + j * H + o0 + rr;
-        const float v = fmaf(R.sigma, msm[rr * rs + j], __ldg(pm + q));
-        cm[q] = v;
-        msm[rr * rs + j] = v;
+      float mx = 0.0f;
+#pragma unroll
+      for (int k = 0; k < kHeld; ++k) {
+        const int idx = tid + k * nt;
+        if (idx < nel) {
+          const int j = idx >> rlog;
+          v[k] = fmaf(R.sigma, msm[rr0 * rs + j], v[k]);
+          cm[q0 + j * H] = v[k];
+          mx = fmaxf(mx, fabsf(v[k]));
+        }
       }
-      __syncthreads();
+      for (int idx = tid + kHeld * nt; idx < nel; idx += nt) {
+        const int j = idx >> rlog;
+        const float w1 = fmaf(R.sigma, msm[rr0 * rs + j], __ldg(pm + q0 + j * H));
+        cm[q0 + j * H] = w1;
+        msm[rr0 * rs + j] = w1;
+        mx = fmaxf(mx, fabsf(w1));
+      }
       if (R.precision == PREC_BF16) {
         __nv_bfloat16 *qw = reinterpret_cast<__nv_bfloat16 *>(cq);
-        for (int idx = tid; idx < nel; idx += nt) {
-          const int j = idx >> kMutRowsLog2, rr = idx & (kMutRows - 1);
-          qw[qbase + j * H + o0 + rr] = __float2bfloat16_rn(msm[rr * rs + j]);
-        }
-      } else if (R.precision == PREC_FP8) {
-        for (int rr = warp; rr < kMutRows; rr += nw) {
-          float mx = 0.0f;
-          for (int j = lane; j < nin; j += 32) mx = fmaxf(mx, fabsf(msm[rr * rs + j]));
 #pragma unroll
-          for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, off));
-          float s = __fdiv_rn(mx, 448.0f);
-          if (s == 0.0f) s = 1.0f;
-          if (lane == 0) {
-            s_scale[rr] = s;
-            reinterpret_cast<float *>(cq + L.off_scale)[srow + o0 + rr] = s;
-          }
+        for (int k = 0; k < kHeld; ++k) {
+          const int idx = tid + k * nt;
+          if (idx < nel) qw[q0 + (idx >> rlog) * H] = __float2bfloat16_rn(v[k]);
         }
+        for (int idx = tid + kHeld * nt; idx < nel; idx += nt)
+          qw[q0 + (idx >> rlog) * H] = __float2bfloat16_rn(msm[rr0 * rs + (idx >> rlog)]);
+      } else if (R.precision == PREC_FP8) {
+        // the rows' maxima (non-negative floats compare as their bits): lanes
+        // `rows` apart hold the same row
+        for (int off = rows; off < 32; off <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, off));
+        if (lane < rows) atomicMax(&s_max[lane], __float_as_uint(mx));
         __syncthreads();
-        for (int idx = tid; idx < nel; idx += nt) {
-          const int j = idx >> kMutRowsLog2, rr = idx & (kMutRows - 1);
-          cq[qbase + j * H + o0 + rr] = e4m3_sat(__fdiv_rn(msm[rr * rs + j], s_scale[rr]));
+        float sc = __fdiv_rn(__uint_as_float(s_max[rr0]), 448.0f);
+        if (sc == 0.0f) sc = 1.0f;
+        if (tid < rows) reinterpret_cast<float *>(cq + L.off_scale)[srow + o0 + rr0] = sc;
+#pragma unroll
+        for (int k = 0; k < kHeld; ++k) {
+          const int idx = tid + k * nt;
+          if (idx < nel) cq[q0 + (idx >> rlog) * H] = e4m3_sat(__fdiv_rn(v[k], sc));
+        }
+        for (int idx = tid + kHeld * nt; idx < nel; idx += nt) {
+          const int j = idx >> rlog;
+          cq[q0 + j * H] = e4m3_sat(__fdiv_rn(msm[rr0 * rs + j], sc));
         }
       }
       __syncthreads();
@@ -932,35 +961,94 @@ __device__ void ph_mutate(const Dev &d, const Layout &L, const Rules &R, int b0,
 }
 
 // The mutation in the persistent kernel, FP32 and BF16 forms (FP8 needs
-// each row's maximum first and keeps ph_mutate's tiles): every parameter of
-// every child is an independent element -- its normal comes from the
-// Philox block of its logical index, as in ph_mutate -- so the grid's
-// threads (g0, stride gs) take elements across children and layers with
-// no block barrier between tiles.  The same draws and fmaf as ph_mutate,
-// so the same values bit for bit; each element draws its own Philox block
-// (four times the arithmetic of the tiled form, which the tiles' barriers
-// and dependent loads outweigh).
+// each row's maximum first and keeps ph_mutate's tiles), without a block
+// barrier.  The same draws and fmaf as ph_mutate, so the same values bit for
+// bit.
+//
+// One element: its normal comes from the Philox block of its logical index
+// (four times the arithmetic of the tiled form).
+__device__ __forceinline__ void put_child(const Layout &L, const Rules &R, float *cm, uint8_t *cq, int q, float v) {
+  cm[q] = v;
+  if (R.precision == PREC_BF16) {
+    if (q < L.nW)
+      reinterpret_cast<__nv_bfloat16 *>(cq)[q] = __float2bfloat16_rn(v);
+    else
+      reinterpret_cast<float *>(cq + L.off_bias)[q - L.nW] = v;
+  }
+}
+
+__device__ __forceinline__ void mutate_element(const Dev &d, const Layout &L, const Rules &R, uint32_t t, int2 pc, int q) {
+  const int64_t mper = L.mstride / 4;
+  const EnvDesc ed = d.env[env_index(d, pc.y)];
+  const int p = layout_logical(L, q);
+  const U4 r = philox(t, (uint32_t)(pc.x - ed.slot_off), (uint32_t)(p >> 2), 0u, ed.seed, S_MUTATE);
+  const float v = fmaf(R.sigma, normal_of(r, p & 3), __ldg(d.master + (int64_t)pc.x * mper + q));
+  put_child(L, R, d.master + (int64_t)pc.y * mper, d.wq + (int64_t)pc.y * L.stride, q, v);
+}
+
+// While a step's births have no more parameters than the grid has threads,
+// every parameter is an independent element, on as few CTAs as they fill
+// (cta counts from those with nothing else to do).  Beyond, the arithmetic
+// counts: a lane takes kRun consecutive inputs of one output row, at most 11
+// normals from three blocks, 32 rows side by side, so that the masters go
+// through in whole lines, and the runs spread over all CTAs.
+// 371-64-64-9 BF16, us from the last barrier to the step's end, medians: 10
+// to 19 claimants 9.3 -> 8.0, 20 to 39 claimants 11.5 -> 8.5, elements -> runs.
+constexpr int kRun = 8;
+
 __device__ void ph_mutate_flat(const Dev &d, const Layout &L, const Rules &R, uint32_t t, const int *par,
-                               const int *chi, int nbirths, int g0, int gs) {
+                               const int *chi, int nbirths, int cta, int ctas) {
   const int nb = par ? nbirths : d.counters[CNT_N_BIRTHS];
   const int P = L.nW + L.nB;  // physical master elements: weights, then biases (and tau)
+  const int gs = ctas * (int)blockDim.x;
+  auto pair_of = [&](int b) { return par ? make_int2(par[b], chi[b]) : d.births[b]; };
+  if ((long long)nb * P <= gs) {
+    const int w = cta * (int)blockDim.x + (int)threadIdx.x;
+    if (w < nb * P) mutate_element(d, L, R, t, pair_of(w / P), w - w / P * P);
+    return;
+  }
+  const int D = L.D, H = L.H, lane = threadIdx.x & 31;
   const int64_t mper = L.mstride / 4;
-  for (int w = g0; w < nb * P; w += gs) {
-    const int b = w / P, q = w - b * P;
-    const int2 pc = par ? make_int2(par[b], chi[b]) : d.births[b];
+  // warps take pieces of W_in, of the hidden layers, then 32 single elements
+  // of the head and the biases
+  const int in1 = (D + kRun - 1) / kRun, inh = H / kRun;
+  const int pieces_in = H / 32 * in1, pieces_h = H / 32 * inh, pieces_w = pieces_in + L.L * pieces_h;
+  const int q3 = D * H + L.L * H * H;
+  const int pieces = pieces_w + (P - q3 + 31) / 32;
+  for (int w = ((int)threadIdx.x >> 5) * ctas + cta; w < nb * pieces; w += gs >> 5) {
+    const int b = w / pieces, it = w - b * pieces;
+    const int2 pc = pair_of(b);
+    if (it >= pieces_w) {
+      const int q = q3 + 32 * (it - pieces_w) + lane;
+      if (q < P) mutate_element(d, L, R, t, pc, q);
+      continue;
+    }
     const EnvDesc ed = d.env[env_index(d, pc.y)];
     const uint32_t lp = (uint32_t)(pc.x - ed.slot_off);
-    const int p = layout_logical(L, q);
-    const U4 r = philox(t, lp, (uint32_t)(p >> 2), 0u, ed.seed, S_MUTATE);
-    const float v = fmaf(R.sigma, normal_of(r, p & 3), __ldg(d.master + (int64_t)pc.x * mper + q));
-    d.master[(int64_t)pc.y * mper + q] = v;
-    if (R.precision == PREC_BF16) {
-      uint8_t *cq = d.wq + (int64_t)pc.y * L.stride;
-      if (q < L.nW)
-        reinterpret_cast<__nv_bfloat16 *>(cq)[q] = __float2bfloat16_rn(v);
-      else
-        reinterpret_cast<float *>(cq + L.off_bias)[q - L.nW] = v;
-    }
+    const float *pm = d.master + (int64_t)pc.x * mper;
+    float *cm = d.master + (int64_t)pc.y * mper;
+    uint8_t *cq = d.wq + (int64_t)pc.y * L.stride;
+    const bool l1 = it < pieces_in;
+    const int layer = l1 ? 0 : (it - pieces_in) / pieces_h;  // hidden layer
+    const int x = l1 ? it : it - pieces_in - layer * pieces_h;
+    const int nin = l1 ? D : H, chunks = l1 ? in1 : inh;
+    const int row = x / chunks, j0 = (x - row * chunks) * kRun, o = 32 * row + lane;
+    const int nj = min(kRun, nin - j0);
+    const int q = (l1 ? 0 : D * H + layer * H * H) + j0 * H + o;
+    const int p = (l1 ? 0 : D * H + L.ns * H + layer * (H * H + H)) + o * nin + j0;
+    float v[kRun], n[12];
+#pragma unroll
+    for (int k = 0; k < kRun; ++k) v[k] = k < nj ? __ldg(pm + q + k * H) : 0.0f;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) normals4(philox(t, lp, (uint32_t)((p >> 2) + k), 0u, ed.seed, S_MUTATE), n + 4 * k);
+    // the run starts p % 4 normals into the first block
+#pragma unroll
+    for (int k = 0; k < 11; ++k) n[k] = (p & 1) ? n[k + 1] : n[k];
+#pragma unroll
+    for (int k = 0; k < kRun; ++k) n[k] = (p & 2) ? n[k + 2] : n[k];
+#pragma unroll
+    for (int k = 0; k < kRun; ++k)
+      if (k < nj) put_child(L, R, cm, cq, q + k * H, fmaf(R.sigma, n[k], v[k]));
   }
 }
 
@@ -1405,8 +1493,8 @@ __global__ void __launch_bounds__(1024) k_birth_assign(Dev d, Rules R) {
 }
 __global__ void __launch_bounds__(256) k_mutate(Dev d, Layout L, Rules R) {
   extern __shared__ __align__(16) float msm[];
-  __shared__ float s_scale[kMutRows];
-  ph_mutate(d, L, R, blockIdx.x, gridDim.x, msm, s_scale, STEP_T, nullptr, nullptr, 0);
+  __shared__ uint32_t s_max[kMutRows];
+  ph_mutate(d, L, R, blockIdx.x, gridDim.x, msm, s_max, STEP_T, nullptr, nullptr, 0);
 }
 __global__ void k_regrow(Dev d, Rules R) { ph_regrow(d, R, GRID_ARGS, STEP_T, 0u, 0); }
 __global__ void k_flow_out(Dev d) { ph_flow_out(d, GRID_ARGS); }
@@ -1583,7 +1671,7 @@ template <bool CLUSTER>
 __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rules R) {
   extern __shared__ __align__(16) float msm[];
   __shared__ BirthSmem S;
-  __shared__ float s_scale[kMutRows];
+  __shared__ uint32_t s_max[kMutRows];
   __shared__ int s_flag;
   const unsigned nb = gridDim.x;
   const int g0 = blockIdx.x * blockDim.x + threadIdx.x, gs = gridDim.x * blockDim.x;
@@ -1758,9 +1846,9 @@ __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rul
   if (claimants > 0) {
     if (R.precision != PREC_FP8)
       ph_mutate_flat(d, L, R, t, fast ? S.win : nullptr, fast ? S.free_ : nullptr, fast ? S.nborn : 0,
-                     (int)((gridDim.x - 1 - blockIdx.x) * blockDim.x + threadIdx.x), (int)(gridDim.x * blockDim.x));
+                     (int)(nb - 1u - blockIdx.x), (int)nb);
     else
-      ph_mutate(d, L, R, gridDim.x - 1 - blockIdx.x, gridDim.x, msm, s_scale, t, fast ? S.win : nullptr,
+      ph_mutate(d, L, R, gridDim.x - 1 - blockIdx.x, gridDim.x, msm, s_max, t, fast ? S.win : nullptr,
                 fast ? S.free_ : nullptr, fast ? S.nborn : 0);
   }
   if (trow) {
