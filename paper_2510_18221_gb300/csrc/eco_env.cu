@@ -802,6 +802,7 @@ __device__ void ph_birth_assign(const Dev &d, const Rules &R, int b0, int bs, Bi
 // tiles always of 8 rows that went through shared memory three times: 4 to 9
 // claimants (3,400 agents) 9.8 -> 7.9, 20 to 39 (12,000) 20.8 -> 18.0; 1 to 3
 // among 12,000 agents, bound by cold code and masters, 12.0 as before.
+// ---------------------------------------------------------------------------
 constexpr int kMutRows = 8;
 constexpr int kMutRowsLog2 = 3;
 static_assert((1 << kMutRowsLog2) == kMutRows, "kMutRows is a power of two");
@@ -1646,12 +1647,11 @@ __device__ void fast_births(const Dev &d, BirthSmem &S, int nc) {
   __syncthreads();
 }
 
-// Request a plane into L2: 2 KB pieces, consecutive ones by different CTAs
-// (c of n; one SM alone asks for 50 GB/s).
-__device__ __forceinline__ void prefetch_cells(const void *plane, long long bytes, int c, int n) {
+// Request a plane into L2: 2 KB pieces, consecutive ones by different warps
+// (w of n), which lie in different CTAs (one SM alone asks for 50 GB/s).
+__device__ __forceinline__ void prefetch_cells(const void *plane, long long bytes, int w, int n) {
   constexpr long long kPiece = 2048;
-  for (long long at = ((long long)threadIdx.x * n + c) * kPiece; at < (bytes & ~15ll);
-       at += (long long)blockDim.x * n * kPiece) {
+  for (long long at = ((long long)(threadIdx.x & 31) * n + w) * kPiece; at < (bytes & ~15ll); at += 32ll * n * kPiece) {
     const long long left = (bytes & ~15ll) - at;
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(reinterpret_cast<const uint8_t *>(plane) + at),
                  "r"((uint32_t)(left < kPiece ? left : kPiece))
@@ -1674,7 +1674,15 @@ __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rul
   __shared__ uint32_t s_max[kMutRows];
   __shared__ int s_flag;
   const unsigned nb = gridDim.x;
-  const int g0 = blockIdx.x * blockDim.x + threadIdx.x, gs = gridDim.x * blockDim.x;
+  // Consecutive warps' worth of agents go to different CTAs: an agent's cells
+  // lie anywhere, 32 lines to a warp's load, and with CTAs filled one after
+  // the other (1,024 agents on each of a few SMs) an SM's L1 was what a phase
+  // waited for.  Arrival at the first barrier, us: mid FP32 4.1 -> 2.3, paper 4.1
+  // -> 3.1, terrain 5.4 -> 4.5; the step's end without births: mid FP8 18.6 ->
+  // 16.1, paper 17.3 -> 15.7, ecology 19.1 -> 18.1, terrain 33.1 -> 31.2.
+  const int lane = threadIdx.x & 31, n_warps = (int)(nb * (blockDim.x >> 5));
+  const int wk = (int)((threadIdx.x >> 5) * nb + blockIdx.x);
+  const int g0 = 32 * wk + lane, gs = 32 * n_warps;
   // The launch's first reads, issued together: the step, the failure-
   // detection test words (0 unless armed by eco_arm_barrier_timeout,
   // cleared by eco_reset: a CTA that leaves before its first barrier, and the
@@ -1739,19 +1747,17 @@ __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rul
     if (trow && blockIdx.x == 0 && threadIdx.x == 0) trow[TR_PASS0 + bar - 1] = global_ns();
     return ok;
   };
-  // Housekeeping goes to CTAs with little else to do in its interval: the
-  // per-agent phases take one agent per thread from CTA 0 on, and the
-  // alive list's tiles go to CTAs 0 .. tiles - 1.  The cells' phases leave
-  // the CTAs with agents out where those are at most half and the others
-  // have at most four groups a thread (a 2048 x 2048 world or a large batch
-  // has more, and needs every SM).
-  const int agent_ctas = (n_alive + (int)blockDim.x - 1) / (int)blockDim.x;
-  const int rest = (int)nb - agent_ctas;
-  const int cell_first =
-      rest >= agent_ctas && (d.total_cells >> 2) <= 4ll * rest * (int)blockDim.x ? agent_ctas : 0;
+  // The cells' phases leave the warps with agents out where those are at most
+  // half and the others have at most four groups a thread (a 2048 x 2048 world
+  // or a large batch has more, and needs every warp).
+  const int agent_warps = min((n_alive + 31) / 32, n_warps);
+  const int rest = n_warps - agent_warps;
+  const int cell_first = rest >= agent_warps && (d.total_cells >> 2) <= 128ll * rest ? agent_warps : 0;
   const int regrow_ahead = cell_first > 0 && d.n_envs == 1 ? kRegrowAhead : 0;
-  const int cg0 = g0 - cell_first * (int)blockDim.x, cgs = gs - cell_first * (int)blockDim.x;
-  const bool cell_cta = (int)blockIdx.x >= cell_first;
+  const int cg0 = g0 - 32 * cell_first, cgs = gs - 32 * cell_first;
+  const bool cell_warp = wk >= cell_first;
+  // Housekeeping goes to CTAs without the alive list's tiles, which are on
+  // CTAs 0 .. tiles - 1.
   const int tiles = compact_tiles(d.total_slots);
   const unsigned last = nb - 1u;
   const unsigned fold_cta = (unsigned)tiles < nb ? (unsigned)tiles : 0u;      // statistics
@@ -1767,13 +1773,13 @@ __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rul
   Agent ag;
   uint32_t draws = 0u;
   ph_move_apply_eat(d, R, L.A, g0, gs, first, t, ag);
-  if (cell_cta) {
+  if (cell_warp) {
     if (R.rules != RULES_TERRAIN) {
       if (regrow_ahead) draws = regrow_draws(d, R, cg0, cgs, t);
     } else {
       // the policy kernel's weight stream has pushed the cells' planes out of
       // L2: bring them back ahead of the cells' phases
-      const int cc = (int)blockIdx.x - cell_first, ncc = (int)nb - cell_first;
+      const int cc = wk - cell_first, ncc = n_warps - cell_first;
       prefetch_cells(d.cellf, d.total_cells, cc, ncc);
       prefetch_cells(d.bio, 4 * (long long)d.total_cells, cc, ncc);
       prefetch_cells(d.res, 4 * (long long)d.total_cells, cc, ncc);
@@ -1785,7 +1791,7 @@ __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rul
   if (!sync()) return;
   ph_metab_death(d, R, g0, gs, t, ag);
   // simple rules: only eating takes food, and it is over
-  if (R.rules == RULES_SIMPLE && cell_cta) ph_regrow(d, R, cg0, cgs, t, draws, regrow_ahead);
+  if (R.rules == RULES_SIMPLE && cell_warp) ph_regrow(d, R, cg0, cgs, t, draws, regrow_ahead);
   if (!sync()) return;
   // regrowth under the other rules (with photosynthesis and the flow's
   // transfers) needs the state after the deaths, and birth claims read only
@@ -1795,8 +1801,8 @@ __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rul
   if (d.n_envs == 1 && compact_tiles(d.total_slots) <= kMaxFastTiles) list_free_slots(d, S.sh);
   TileScan ts = {0u, 0, 0, 0};
   if (tiles <= (int)nb && (int)blockIdx.x < tiles) ts = compact_scan(d, blockIdx.x, S.sh64, t);
-  if (R.rules != RULES_SIMPLE && cell_cta) ph_regrow(d, R, cg0, cgs, t, draws, regrow_ahead);
-  if (R.rules == RULES_TERRAIN && cell_cta) ph_flow_out(d, cg0, cgs);
+  if (R.rules != RULES_SIMPLE && cell_warp) ph_regrow(d, R, cg0, cgs, t, draws, regrow_ahead);
+  if (R.rules == RULES_TERRAIN && cell_warp) ph_flow_out(d, cg0, cgs);
   if (!sync()) return;
   // Every claim is in, and the count of claimants does not change again
   // in this launch, so every CTA takes the same branch.
