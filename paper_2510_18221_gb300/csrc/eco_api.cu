@@ -568,7 +568,9 @@ static int check_status(eco_handle *h) {
 static int make_list(eco_handle *h) {
   if (h->list_current) return ECO_OK;
   CUDA_TRY(h, launch_compact(h->d, h->stream));
-  h->list_current = true;
+  cudaStreamCaptureStatus cap;  // a captured launch has not run yet
+  CUDA_TRY(h, cudaStreamIsCapturing(h->stream, &cap));
+  h->list_current = cap == cudaStreamCaptureStatusNone;
   return ECO_OK;
 }
 

@@ -1557,8 +1557,8 @@ __device__ bool grid_sync(unsigned *count, int *status_word, unsigned nblocks, u
 // compaction tile of 4096 slots (at most kFastBirths, env-local, ascending)
 // into free_list[tile * kFastBirths + i], and the tile's free count into
 // free_tiles[tile]; once the deaths are final and before any birth.  Tile k
-// is scanned by CTA nb - 1 - k (the last CTAs have the least grid-stride
-// work in the birth-claim interval), four slots per thread.
+// is scanned by CTA nb - 1 - k (the first CTAs scan the alive list's tiles
+// in the same interval), four slots per thread.
 __device__ void list_free_slots(const Dev &d, int *sh) {
   const int n = d.env[0].n_slots;
   const int tiles = (n + kCompactTile - 1) / kCompactTile;
@@ -1705,14 +1705,16 @@ __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rul
                  cuda::memory_order_relaxed) & kStatusTimeout;
   }
   __syncthreads();
+  // the host's copy of a step that stops early, which no fold will write:
+  // everything as it stands (every CTA writes the same words)
+  auto mirror_all = [&]() {
+    const int words = (int)(reinterpret_cast<const int32_t *>(d.counters + CNT_N) -
+                            reinterpret_cast<const int32_t *>(d.stats_total));
+    for (int i = threadIdx.x; i < words; i += blockDim.x)
+      reinterpret_cast<int32_t *>(d.mirror)[i] = reinterpret_cast<const int32_t *>(d.stats_total)[i];
+  };
   if (s_flag) {
-    // the host's copy, which no fold will write: everything as it stands
-    if (d.mirror && blockIdx.x == 0) {
-      const int words = (int)(reinterpret_cast<const int32_t *>(d.counters + CNT_N) -
-                              reinterpret_cast<const int32_t *>(d.stats_total));
-      for (int i = threadIdx.x; i < words; i += blockDim.x)
-        reinterpret_cast<int32_t *>(d.mirror)[i] = reinterpret_cast<const int32_t *>(d.stats_total)[i];
-    }
+    if (d.mirror && blockIdx.x == 0) mirror_all();
     return;
   }
   if (absent == blockIdx.x + 1u) return;
@@ -1743,7 +1745,11 @@ __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rul
     } else {
       ok = grid_sync(count, d.counters + CNT_STATUS, nb, budget, bar, &s_flag);
     }
-    if (!ok && d.mirror && threadIdx.x == 0) *mirror_of(d, d.counters + CNT_STATUS) = kStatusTimeout;
+    if (!ok && d.mirror) {
+      mirror_all();
+      __syncthreads();
+      if (threadIdx.x == 0) *mirror_of(d, d.counters + CNT_STATUS) = kStatusTimeout;
+    }
     if (trow && blockIdx.x == 0 && threadIdx.x == 0) trow[TR_PASS0 + bar - 1] = global_ns();
     return ok;
   };

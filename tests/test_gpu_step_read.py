@@ -49,3 +49,20 @@ def test_timeout_reaches_a_pipelined_read():
     before = eco.eco_step_read(env.h, 1)[0][0]
     assert before[0] == 0 and eco.eco_read_stats(env.h, 1)[0][0][0] == 1
     env.close()
+
+
+def test_records_of_a_step_that_timed_out():
+    """The read that reports a timeout still hands over the records as the
+    stopped step left them: those of the step before it."""
+    from paper_2510_18221_gb300 import eco
+    env = eco.Env(workloads.scaled("mid", 128, 8192, 4000, precision="bf16"))
+    env.reset()
+    for _ in range(3):
+        eco.eco_step_read(env.h, 1)
+    want = eco.eco_read_stats(env.h, 1)
+    eco.eco_arm_barrier_timeout(env.h, env.launch_mode()[1] - 1, 100000)
+    eco.eco_step_read(env.h, 1)
+    total, last = np.zeros((2, 1, eco.ECO_N_STATS), np.int64)
+    rc = eco.lib().eco_step_read(env.h, total.ctypes.data, last.ctypes.data, 1)
+    assert rc == eco.ECO_ETIMEOUT
+    assert np.array_equal(total, want[0]) and np.array_equal(last, want[1])
