@@ -27,7 +27,19 @@
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
 
+#include <mutex>
+
 namespace eco {
+
+cudaError_t allow_dynamic_smem(const void *kernel, size_t bytes) {
+  static std::mutex mutex;  // two threads raising one limit: the larger value stays
+  std::lock_guard<std::mutex> lock(mutex);
+  cudaFuncAttributes a;
+  const cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+  if (e != cudaSuccess) return e;
+  if (a.maxDynamicSharedSizeBytes >= 0 && (size_t)a.maxDynamicSharedSizeBytes >= bytes) return cudaSuccess;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
 
 int grid_for(long long n, int threads, int max_blocks) {
   long long b = (n + threads - 1) / threads;
@@ -1884,12 +1896,11 @@ cudaError_t launch_compact(const Dev &d, cudaStream_t s) {
 
 cudaError_t env_prepare(const Layout &L, EnvGrid *g) {
   const size_t smem = mutate_smem_bytes(L);
-  cudaError_t e = cudaFuncSetAttribute((const void *)k_mutate, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  cudaError_t e = allow_dynamic_smem((const void *)k_mutate, smem);
   if (e != cudaSuccess) return e;
   const void *const forms[2] = {(const void *)k_env_persistent<false>, (const void *)k_env_persistent<true>};
   for (const void *f : forms)
-    if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+    if ((e = allow_dynamic_smem(f, smem)) != cudaSuccess) return e;
   int dev = 0, coop = 0, per_sm = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev)) != cudaSuccess) return e;

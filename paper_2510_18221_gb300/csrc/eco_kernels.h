@@ -50,6 +50,13 @@ struct EnvGrid {
   int cluster;            // the persistent form's CTAs are one thread-block cluster
 };
 __host__ __device__ int compact_tiles(int total_slots);
+
+// Let `kernel` be launched with `bytes` of dynamic shared memory.  The limit
+// belongs to the function on the device, not to a handle, so it is only ever
+// raised: a handle of a smaller shape leaves a larger one's launches their
+// room.  Safe from several host threads.
+cudaError_t allow_dynamic_smem(const void *kernel, size_t bytes);
+
 // Alive list of the current state (ascending slots) and its count.
 cudaError_t launch_compact(const Dev &d, cudaStream_t s);
 // Shared-memory attributes and the persistent form's grid size.

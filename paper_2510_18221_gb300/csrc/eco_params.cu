@@ -334,7 +334,7 @@ static cudaError_t launch_tiled(K *kernel, const Dev &d, const Layout &L, int sl
   int rlog = 3;
   while ((1 << rlog) < rows) ++rlog;
   const size_t smem = tile_bytes(L, rows);
-  cudaError_t e = cudaFuncSetAttribute((const void *)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_dynamic_smem((const void *)kernel, smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0, per_sm = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;

@@ -69,7 +69,7 @@ cudaError_t policy_prepare(const Layout &L, const Rules &R, int variant, PolicyL
   }
   const void *fn = (const void *)pick(R.precision, L.H, variant);
   if (!fn) return cudaErrorInvalidValue;
-  e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = allow_dynamic_smem(fn, smem);
   if (e != cudaSuccess) return e;
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
