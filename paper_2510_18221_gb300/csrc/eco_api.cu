@@ -10,6 +10,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <vector>
 
 #include "../../include/eco.h"
@@ -76,6 +77,10 @@ struct eco_handle {
   cudaEvent_t rd_ev[2];
   uint8_t *bounce;  // pinned, behind rd_host's slots: a small world's whole state
   size_t bounce_bytes;
+  // held by the calls that pass data through the workspace's staging region
+  // or `bounce`, so that several host threads may read and write states and
+  // parameters of one handle
+  std::mutex io;
   char err[512];
 };
 
@@ -977,6 +982,7 @@ extern "C" int eco_read_state(eco_handle *h, int32_t env, eco_state_view *out) {
   int rc = check_env(h, env);
   if (rc) return rc;
   if (!out) return fail(h, ECO_EINVAL, "null view");
+  std::lock_guard<std::mutex> io(h->io);
   const EnvDesc &ed = h->env_host[env];
   const size_t N = (size_t)ed.side * ed.side, S = (size_t)ed.n_slots;
   const Dev &d = h->d;
@@ -1197,6 +1203,7 @@ extern "C" int eco_read_params(eco_handle *h, int32_t env, int32_t slot0, int32_
   if (rc) return rc;
   if (n == 0) return ECO_OK;
   if (!out) return fail(h, ECO_EINVAL, "null output");
+  std::lock_guard<std::mutex> io(h->io);
   // the device puts a chunk of slots into logical order, then one copy takes
   // it to the caller (a host loop over the elements ran at 4 GB/s)
   const int g0 = h->env_host[env].slot_off + slot0;
@@ -1216,6 +1223,7 @@ extern "C" int eco_write_params(eco_handle *h, int32_t env, int32_t slot0, int32
   if (rc) return rc;
   if (n == 0) return ECO_OK;
   if (!in) return fail(h, ECO_EINVAL, "null input");
+  std::lock_guard<std::mutex> io(h->io);
   const int g0 = h->env_host[env].slot_off + slot0;
   const size_t P = (size_t)h->L.P;
   for (int a = 0; a < n; a += h->d.staging_slots) {
