@@ -232,9 +232,13 @@ static Layout make_layout(const eco_config *c) {
   return L;
 }
 
-// The parameter staging region holds about this many bytes (one slot at
-// least): transfers of 32 MB run at the host link's rate.
+// The staging region of state and parameter transfers is at most about this
+// many bytes (but holds one slot's parameters): transfers of 32 MB run at the
+// host link's rate.  It need not exceed the largest transfer of the handle.
 constexpr long long kStagingBytes = 32ll << 20;
+// Bytes per cell (food, wall, occupant) and per slot (x, y, RGB) of the arrays
+// of eco_read_state that a kernel converts in the staging region.
+constexpr long long kCellOut = 6, kSlotOut = 20;
 // Worlds whose whole state fits this are read through pinned memory.
 constexpr size_t kBounceBytes = 1u << 20;
 // Bytes of every array of eco_read_state for N cells and S slots, each padded
@@ -258,11 +262,16 @@ struct Carve {
 static size_t carve(const eco_config *c, const Layout &L, uint8_t *base, Dev *d, EnvDesc **env_dev) {
   Carve k;
   k.base = base;
-  long long cells = 0, slots = 0, ctiles = 0;
+  long long cells = 0, slots = 0, ctiles = 0, state = 0;
   for (int e = 0; e < c->n_envs; ++e) {
     cells += (long long)c->env_side[e] * c->env_side[e];
     slots += c->env_slots[e];
     ctiles += place_tiles(c->env_side[e]);
+    // what eco_read_state holds at a time: a small world's whole state, else
+    // the converted cells, then the converted slots
+    const long long n = (long long)c->env_side[e] * c->env_side[e], s = c->env_slots[e];
+    const long long whole = (long long)state_bytes((size_t)n, (size_t)s);
+    state = std::max({state, kCellOut * n, kSlotOut * s, whole <= (long long)kBounceBytes ? whole : 0ll});
   }
   const int E = c->n_envs;
   Dev &D = *d;
@@ -331,8 +340,12 @@ static size_t carve(const eco_config *c, const Layout &L, uint8_t *base, Dev *d,
   D.a_water = k.take<int32_t>(slots);
   D.a_bio = k.take<int32_t>(slots);
   D.trace = k.take<unsigned long long>((size_t)kTraceSteps * kTraceWords);
-  D.staging_slots = (int)std::min(slots, std::max(1ll, kStagingBytes / (4ll * L.P)));
-  D.staging = k.take<float>((size_t)D.staging_slots * L.P);
+  const long long slot_bytes = 4ll * L.P;
+  D.staging_slots = (int)std::min(slots, std::max(1ll, kStagingBytes / slot_bytes));
+  // (with the slots' parameters alone, a 1024 x 1024 world of 4 slots was read
+  // in 170 pieces: 6.3 ms against 0.8)
+  D.staging_bytes = (size_t)std::max(D.staging_slots * slot_bytes, std::min(kStagingBytes, state));
+  D.staging = reinterpret_cast<float *>(k.take<uint8_t>(D.staging_bytes));
   // The policy kernel's FP8 tail batches and its requests into L1 reach up
   // to kStreamSlack bytes past the last weight block (no product uses them):
   // the regions after the weights (the histogram alone is 256 KB per world)
@@ -1002,8 +1015,8 @@ extern "C" int eco_read_state(eco_handle *h, int32_t env, eco_state_view *out) {
                {out->photo, d.photo + co, 4 * N},    {out->step, d.step, sizeof(int64_t)}};
   // arrays a kernel converts: every cell's food, wall and env-local occupant
   // (6 bytes a cell), every slot's x, y and RGB (20 bytes a slot)
-  const size_t staging = (size_t)d.staging_slots * h->L.P * 4;
-  if (state_bytes(N, S) <= std::min(h->bounce_bytes, staging)) {
+  const size_t staging = d.staging_bytes;
+  if (state_bytes(N, S) <= kBounceBytes) {
     // a small world: everything packed by one kernel and brought over by one
     // copy into pinned memory (a copy per array cost 0.3 ms)
     uint8_t *base = reinterpret_cast<uint8_t *>(d.staging);
@@ -1040,7 +1053,7 @@ extern "C" int eco_read_state(eco_handle *h, int32_t env, eco_state_view *out) {
   };
   // converted arrays in pieces of the staging region, a multiple of 4 cells
   uint8_t *base = reinterpret_cast<uint8_t *>(d.staging);
-  const size_t cell_piece = std::max<size_t>(4, staging / 6 / 4 * 4), slot_piece = std::max<size_t>(1, staging / 20);
+  const size_t cell_piece = staging / kCellOut / 4 * 4, slot_piece = staging / kSlotOut;
   if (out->food || out->wall || out->occ)
     for (size_t c = 0; c < N; c += cell_piece) {
       const size_t n = std::min(cell_piece, N - c);
