@@ -961,6 +961,12 @@ extern "C" int eco_step_read(eco_handle *h, eco_stats *total, eco_stats *last, i
   const int slot = prev == 1 ? 2 : 1;
   int rc = build_graph(h, slot == 1 ? GRAPH_READ1 : GRAPH_READ2);
   if (rc) return rc;
+  // nothing that writes this slot is in flight: its last step was waited for
+  // by the call after it, or by a reset.  The step stores a status other than 0
+  // only (its CTAs' stores come in no order).
+  const size_t status_at = (size_t)(reinterpret_cast<uint8_t *>(h->d.counters + CNT_STATUS) -
+                                    reinterpret_cast<uint8_t *>(h->d.stats_total));
+  memset(h->rd_host + slot * h->rd_bytes + status_at, 0, sizeof(int32_t));
   CUDA_TRY(h, cudaGraphLaunch(h->graph[slot == 1 ? GRAPH_READ1 : GRAPH_READ2], h->stream));
   h->steps_done += 1;
   CUDA_TRY(h, cudaEventRecord(h->rd_ev[slot - 1], h->stream));

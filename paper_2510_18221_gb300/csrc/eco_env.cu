@@ -1471,7 +1471,10 @@ __device__ void fold_env(const Dev &d, const Rules &R, int e, long long t, int b
       *mirror_of(d, tot + k) = v;
     }
   }
-  if (d.mirror && e == 0 && lane == 0) *mirror_of(d, d.counters + CNT_STATUS) = d.counters[CNT_STATUS];
+  // the host's status word is 0 before the launch, and only what is not 0 is
+  // stored: a CTA whose wait ran out stores it too, in no order with this one
+  if (d.mirror && e == 0 && lane == 0 && d.counters[CNT_STATUS] != 0)
+    *mirror_of(d, d.counters + CNT_STATUS) = d.counters[CNT_STATUS];
 }
 
 // ---------------------------------------------------------------------------
@@ -1718,12 +1721,14 @@ __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rul
   }
   __syncthreads();
   // the host's copy of a step that stops early, which no fold will write:
-  // everything as it stands (every CTA writes the same words)
+  // the records as they stand (every CTA writes the same words) and the
+  // timeout
   auto mirror_all = [&]() {
-    const int words = (int)(reinterpret_cast<const int32_t *>(d.counters + CNT_N) -
+    const int words = (int)(reinterpret_cast<const int32_t *>(d.counters) -
                             reinterpret_cast<const int32_t *>(d.stats_total));
     for (int i = threadIdx.x; i < words; i += blockDim.x)
       reinterpret_cast<int32_t *>(d.mirror)[i] = reinterpret_cast<const int32_t *>(d.stats_total)[i];
+    if (threadIdx.x == 0) *mirror_of(d, d.counters + CNT_STATUS) = d.counters[CNT_STATUS] | kStatusTimeout;
   };
   if (s_flag) {
     if (d.mirror && blockIdx.x == 0) mirror_all();
@@ -1757,11 +1762,7 @@ __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rul
     } else {
       ok = grid_sync(count, d.counters + CNT_STATUS, nb, budget, bar, &s_flag);
     }
-    if (!ok && d.mirror) {
-      mirror_all();
-      __syncthreads();
-      if (threadIdx.x == 0) *mirror_of(d, d.counters + CNT_STATUS) = kStatusTimeout;
-    }
+    if (!ok && d.mirror) mirror_all();
     if (trow && blockIdx.x == 0 && threadIdx.x == 0) trow[TR_PASS0 + bar - 1] = global_ns();
     return ok;
   };
