@@ -62,7 +62,8 @@ struct eco_handle {
   // steps run since reset (a host shadow of the device's step counter) and
   // the first step of every timed launch not yet reported
   long long steps_done;
-  bool list_current;  // the alive list is that of the current state
+  // the alive list against the current state (make_list)
+  enum { LIST_STALE, LIST_STEPPED, LIST_CURRENT } list;
   std::vector<long long> timed_steps;
   cudaEvent_t ev_dummy[2];
   std::vector<cudaEvent_t> ev_pool;  // pairs
@@ -497,7 +498,7 @@ extern "C" int eco_create(const eco_config *cfg, void *dev_workspace, size_t byt
   }
   h->ev_used = 0;
   h->steps_done = 0;
-  h->list_current = false;
+  h->list = eco_handle::LIST_STALE;
   h->rd_pending = 0;
   h->rd_ev[0] = h->rd_ev[1] = nullptr;
   h->err[0] = 0;
@@ -580,15 +581,17 @@ static int check_status(eco_handle *h) {
   return ECO_OK;
 }
 
-// The alive list of the current state.  Reset, state writes and every step
-// leave it so: only a handle that has seen none of them still has to make it
-// (eco_policy_only made it on each call, two kernels of 2 us).
+// The alive list of the current state.  Reset and state writes leave it so
+// (eco_policy_only made it on each call, two kernels of 2 us), and so does a
+// step that ran to its end: after steps whose status nobody has read yet the
+// list is made again, since one that timed out leaves the state between two
+// lists.
 static int make_list(eco_handle *h) {
-  if (h->list_current) return ECO_OK;
+  if (h->list == eco_handle::LIST_CURRENT) return ECO_OK;
   CUDA_TRY(h, launch_compact(h->d, h->stream));
   cudaStreamCaptureStatus cap;  // a captured launch has not run yet
   CUDA_TRY(h, cudaStreamIsCapturing(h->stream, &cap));
-  h->list_current = cap == cudaStreamCaptureStatusNone;
+  if (cap == cudaStreamCaptureStatusNone) h->list = eco_handle::LIST_CURRENT;
   return ECO_OK;
 }
 
@@ -597,7 +600,7 @@ extern "C" int eco_reset(eco_handle *h) {
   // also clears the status word, the persistent form's barrier and its
   // failure-detection test words
   CUDA_TRY(h, cudaMemsetAsync(h->d.barrier, 0, BAR_N * sizeof(unsigned), h->stream));
-  h->list_current = false;
+  h->list = eco_handle::LIST_STALE;
   CUDA_TRY(h, launch_reset(h->d, h->L, h->R, h->grid, h->stream));
   const int rc = make_list(h);
   if (rc) return rc;
@@ -759,6 +762,12 @@ static int build_graph(eco_handle *h, int kind) {
   return ECO_OK;
 }
 
+// Steps are about to be enqueued: the list is theirs to keep current, unless
+// one of them times out.
+static void list_stepped(eco_handle *h) {
+  if (h->list == eco_handle::LIST_CURRENT) h->list = eco_handle::LIST_STEPPED;
+}
+
 static int step_impl(eco_handle *h, int32_t n_steps, bool timed) {
   if (!h) return fail(nullptr, ECO_EINVAL, "null handle");
   if (n_steps < 0) return fail(h, ECO_EINVAL, "n_steps < 0");
@@ -768,6 +777,7 @@ static int step_impl(eco_handle *h, int32_t n_steps, bool timed) {
     int rc = many ? build_graph(h, GRAPH_MANY) : ECO_OK;
     if (rc == ECO_OK && rest) rc = build_graph(h, GRAPH_ONE);
     if (rc) return rc;
+    list_stepped(h);
     for (int i = 0; i < many; ++i) CUDA_TRY(h, cudaGraphLaunch(h->graph[GRAPH_MANY], h->stream));
     for (int i = 0; i < rest; ++i) CUDA_TRY(h, cudaGraphLaunch(h->graph[GRAPH_ONE], h->stream));
     h->steps_done += n_steps;
@@ -789,6 +799,7 @@ static int step_impl(eco_handle *h, int32_t n_steps, bool timed) {
     CUDA_TRY(h, cudaEventCreate(&ev));
     h->ev_pool.push_back(ev);
   }
+  list_stepped(h);
   for (int i = 0; i < launches; ++i) {
     CUDA_TRY(h, cudaGraphExecEventRecordNodeSetEvent(gx, h->ev_node[kind][0], h->ev_pool[2 * h->ev_used]));
     CUDA_TRY(h, cudaGraphExecEventRecordNodeSetEvent(gx, h->ev_node[kind][1], h->ev_pool[2 * h->ev_used + 1]));
@@ -931,7 +942,7 @@ static int stats_from_mirror(eco_handle *h, int slot, eco_stats *total, eco_stat
   memcpy(&st, mirror(h->d.counters + CNT_STATUS), sizeof st);
   if (st & 3) return fail(h, ECO_EINVAL, "reset: fewer non-wall cells than founders (status %d)", st);
   if (st & 4) {
-    h->list_current = false;  // the state is partly stepped
+    h->list = eco_handle::LIST_STALE;  // the state is partly stepped
     return fail(h, ECO_ETIMEOUT, "a device-side wait ran out of its budget");
   }
   return ECO_OK;
@@ -944,7 +955,10 @@ extern "C" int eco_read_stats(eco_handle *h, eco_stats *total, eco_stats *last, 
   // memory, one synchronisation, then host-side copies
   CUDA_TRY(h, cudaMemcpyAsync(h->rd_host, h->d.stats_total, h->rd_bytes, cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-  return stats_from_mirror(h, 0, total, last, n_envs);
+  const int rc = stats_from_mirror(h, 0, total, last, n_envs);
+  // every step so far ran to its end
+  if (rc == ECO_OK && h->list == eco_handle::LIST_STEPPED) h->list = eco_handle::LIST_CURRENT;
+  return rc;
 }
 
 extern "C" int eco_step_read(eco_handle *h, eco_stats *total, eco_stats *last, int32_t n_envs) {
@@ -967,6 +981,7 @@ extern "C" int eco_step_read(eco_handle *h, eco_stats *total, eco_stats *last, i
   const size_t status_at = (size_t)(reinterpret_cast<uint8_t *>(h->d.counters + CNT_STATUS) -
                                     reinterpret_cast<uint8_t *>(h->d.stats_total));
   memset(h->rd_host + slot * h->rd_bytes + status_at, 0, sizeof(int32_t));
+  list_stepped(h);
   CUDA_TRY(h, cudaGraphLaunch(h->graph[slot == 1 ? GRAPH_READ1 : GRAPH_READ2], h->stream));
   h->steps_done += 1;
   CUDA_TRY(h, cudaEventRecord(h->rd_ev[slot - 1], h->stream));
@@ -1119,7 +1134,7 @@ extern "C" int eco_write_state(eco_handle *h, int32_t env, const eco_state_view 
         return fail(h, ECO_EINVAL, "slot %d position out of range", i);
       pos[i] = in->y[i] * ed.side + in->x[i];
     }
-    h->list_current = false;
+    h->list = eco_handle::LIST_STALE;
     CUDA_TRY(h, cudaMemcpyAsync(h->d.alive + ed.slot_off, alive.data(), S, cudaMemcpyHostToDevice, s));
     CUDA_TRY(h, cudaMemcpyAsync(h->d.pos + ed.slot_off, pos.data(), 4 * (size_t)S, cudaMemcpyHostToDevice, s));
   }
@@ -1167,7 +1182,7 @@ extern "C" int eco_write_state(eco_handle *h, int32_t env, const eco_state_view 
     CUDA_TRY(h, cudaStreamSynchronize(s));
   }
   CUDA_TRY(h, launch_recount(h->d, h->R, s));
-  h->list_current = false;
+  h->list = eco_handle::LIST_STALE;
   rc = make_list(h);
   if (rc) return rc;
   // the persistent form's arrival counts are kept per step parity, which a
