@@ -18,7 +18,7 @@ LIB = os.path.join(HERE, "libeco.so")
 SOURCES = ["eco_policy_fp8.cu", "eco_policy_bf16.cu", "eco_policy_fp32.cu", "eco_api.cu",
            "eco_policy.cu", "eco_env.cu", "eco_init.cu", "eco_params.cu",
            "eco_noalloc.cu"]
-HEADERS = ["eco_internal.cuh", "eco_kernels.h", "eco_policy_kernel.cuh"]
+HEADERS = ["eco_internal.cuh", "eco_kernels.h", "eco_policy_kernel.cuh", "eco_policy_agents.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
               "--expt-relaxed-constexpr", "-I", os.path.join(ROOT, "include")]

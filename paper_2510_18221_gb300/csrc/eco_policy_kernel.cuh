@@ -757,122 +757,25 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
   // 45.7 -> 39.6).  Where the line lies: 2,400 agents gain from L2 (29.0 -> 23.2)
   // and lose from HBM (35.5 -> 39.6), 4,800 lose in both (45.5 -> 49.3), their
   // stream being bound by bandwidth.
-  const bool few = 8 * n_alive <= 3 * G;
-  const int w0 = few ? warp * (int)gridDim.x + (int)blockIdx.x : (int)blockIdx.x * WARPS + warp;
-  // At the start of the launch every warp gathers an observation with no
-  // weights in flight: the first 4 KB of each warp's first agent's weights
-  // are requested into L2 before that gather.
-  if (lane == 0 && w0 < G_eff && w0 < n_alive)
-    prefetch_l2(d.wq + (int64_t)d.alive_list[w0] * L.stride, (uint32_t)min((int64_t)4096, (int64_t)L.off_w2));
-  // The next agent's slot is read one agent ahead, and its environment,
-  // cell and facing while the current agent's head is computed, so a new
-  // agent starts with its observation gather.  (A slot's facing is written
-  // only by the warp that computes it, in its own iteration.)
-  int i = w0 < G_eff ? w0 : n_alive;
-  // one-hot vision under the simple rules: cells_list's short cut
-  const bool ahead = R.vision == VISION_CHANNELS && R.rules == RULES_SIMPLE && k * k <= 32 * kCellsAhead;
-  int slot_n = 0, env_n = 0, pos_n = 0, f_n = 0;
-  if (i < n_alive) {
-    slot_n = d.alive_list[i];
-    env_n = d.env_of[slot_n];
-    pos_n = d.pos[slot_n];
-    f_n = d.facing[slot_n];
-  }
-  for (; i < n_alive; i += G_eff) {
-    const int slot = slot_n, env = env_n, pos = pos_n, f = f_n;
-    const bool more = i + G_eff < n_alive;
-    if (more) slot_n = d.alive_list[i + G_eff];
-    if (!SPARSE && few) {
-#pragma unroll
-      for (int q = 0; q < kAheadBatches; ++q)
-        prefetch_batch<UNROLL>(reinterpret_cast<const uint4 *>(d.wq + (int64_t)slot * L.stride) + 32 * UNROLL * q, lane);
-    }
-    if (env != e_cur) {
-      flush();
-      e_cur = env;
-    }
-    int nb_cell = 0;
-    uint32_t nb_flags = 0;
-    [[maybe_unused]] short *idx = reinterpret_cast<short *>(ls + 16);
-    [[maybe_unused]] int n_nz = 0;
-    if (SPARSE && ahead) {
-      CellsAhead ca;
-      cells_load(d, R, slot, env, pos, f, lane, kdiv, ca);
-      n_nz = cells_list(R, ca, f, xs, idx, lane);
-      nb_cell = ca.nb_cell;
-      nb_flags = ca.nb_flags;
+  const bool few_now = 8 * n_alive <= 3 * G;
+  // One loop serves both cases, except in the BF16 form of 8 or 16 warps and 4
+  // units in flight (variants 4 and 5): there the second input layer in the
+  // loop cost the full launch 1.7% (46,000 agents 384.8 -> 391.2 us; 12,000
+  // 110.9 -> 114.4; 2,400 31.0 -> 32.9, before the few-agents form -> one loop),
+  // and a loop for each case gives 385.3, 111.6 and 30.8.  In the other
+  // variants two loops are slower (registers: BF16 variant 6 at 12,000 agents
+  // 106.2 -> 108.1, FP8 variant 10 at 46,000 211.4 -> 235.5).
+  if constexpr (PREC == PREC_BF16 && UNROLL == 4 && WARPS >= 8) {
+    if (few_now) {
+      constexpr bool few = true;
+#include "eco_policy_agents.cuh"
     } else {
-      gather_obs(d, L, R, slot, env, pos, f, xs, lane, kdiv, &nb_cell, &nb_flags);
-      if constexpr (SPARSE) {
-        __syncwarp();
-        n_nz = list_nonzero(L.D, xs, idx, lane);
-      }
+      constexpr bool few = false;
+#include "eco_policy_agents.cuh"
     }
-    __syncwarp();
-
-    const uint8_t *blk = d.wq + (int64_t)slot * L.stride;
-    const uint4 *wb = reinterpret_cast<const uint4 *>(blk);
-    const float *bias = reinterpret_cast<const float *>(blk + L.off_bias);
-    const float *scale = reinterpret_cast<const float *>(blk + L.off_scale);
-
-    // -- input layer: act(sum over sensors of (W_s x_s + b_s)) -> hs
-    if constexpr (SPARSE) {
-      layer_in_major<PREC, H, UNROLL, true, false>(wb + L.off_w1 / 16, n_nz, xs, bias, L.ns, scale, hs,
-                                                   lane, L.relu, idx);
-    } else {
-      // one-hot vision: the patch inputs are 0 or 1, exact in f16
-      const int n_exact = R.vision == VISION_CHANNELS ? L.patch : 0;
-      if (few)
-        layer_in_major<PREC, H, UNROLL, false, true>(wb + L.off_w1 / 16, L.D, xs, bias, L.ns, scale, hs, lane,
-                                                     L.relu, nullptr, n_exact);
-      else
-        layer_in_major<PREC, H, UNROLL, false, false>(wb + L.off_w1 / 16, L.D, xs, bias, L.ns, scale, hs, lane,
-                                                      L.relu, nullptr, n_exact);
-    }
-    __syncwarp();
-    // -- hidden layers: h = act(W_l h + b_l), alternating between hs and xs
-    float *cur = hs, *nxt = xs;
-    for (int l = 0; l < L.L; ++l) {
-      layer_in_major<PREC, H, UNROLL, false, false>(wb + (L.off_w2 + l * H * H * L.es) / 16, H, cur,
-                                                    bias + L.ns * H + l * H, 1, scale + H + l * H, nxt,
-                                                    lane, L.relu, nullptr);
-      __syncwarp();
-      float *tmp = cur;
-      cur = nxt;
-      nxt = tmp;
-    }
-
-    if (more) {
-      env_n = d.env_of[slot_n];
-      pos_n = d.pos[slot_n];
-      f_n = d.facing[slot_n];
-    }
-    // -- head: logits = (W_out h [+ b_out]) / exp(tau) (output-major rows of
-    //    H / E units; the temperature only in the paper form)
-    const uint4 *w3 = wb + L.off_w3 / 16;
-    const int U3 = L.A * UPJ;
-    const float *hb = bias + L.ns * H + L.L * H;  // head bias, then tau
-    const float tmul = L.temp ? expf(-__ldg(hb + (L.out_bias ? L.A : 0))) : 1.0f;
-    // the head's groups of 32 units, up to kHeadBatch of them requested
-    // before the first one is reduced
-    constexpr int kHeadBatch = 4;
-    for (int base = 0; base < U3; base += 32 * kHeadBatch) {
-      uint4 hv[kHeadBatch];
-#pragma unroll
-      for (int g = 0; g < kHeadBatch; ++g) {
-        const int u = base + 32 * g + lane;
-        hv[g] = u < U3 ? ldg_stream(w3 + u) : make_uint4(0u, 0u, 0u, 0u);
-      }
-#pragma unroll
-      for (int g = 0; g < kHeadBatch; ++g)
-        if (base + 32 * g < U3)
-          head_group<PREC, H>(hv[g], base + 32 * g + lane, U3, cur, scale + H + L.L * H, hb, L.out_bias,
-                              L.temp, tmul, ls, lane);
-    }
-    __syncwarp();
-
-    sample_and_claim(d, R, L.A, slot, env, pos, f, ls, lane, t, greedy, apply_moves, nb_cell, nb_flags, cnt);
-    __syncwarp();
+  } else {
+    const bool few = few_now;
+#include "eco_policy_agents.cuh"
   }
   flush();
 }
