@@ -39,6 +39,7 @@ struct eco_handle {
   EnvDesc *env_dev;
   uint8_t *ws;
   size_t ws_bytes;
+  size_t staging_bytes;  // of d.staging
   cudaStream_t stream;
   bool own_stream;
   EnvGrid grid;
@@ -260,7 +261,10 @@ struct Carve {
   }
 };
 
-static size_t carve(const eco_config *c, const Layout &L, uint8_t *base, Dev *d, EnvDesc **env_dev) {
+// Returns the workspace's size.  staging_bytes: the staging region's (kept
+// beside Dev, which every kernel takes as a parameter).
+static size_t carve(const eco_config *c, const Layout &L, uint8_t *base, Dev *d, EnvDesc **env_dev,
+                    size_t *staging_bytes) {
   Carve k;
   k.base = base;
   long long cells = 0, slots = 0, ctiles = 0, state = 0;
@@ -345,8 +349,8 @@ static size_t carve(const eco_config *c, const Layout &L, uint8_t *base, Dev *d,
   D.staging_slots = (int)std::min(slots, std::max(1ll, kStagingBytes / slot_bytes));
   // (with the slots' parameters alone, a 1024 x 1024 world of 4 slots was read
   // in 170 pieces: 6.3 ms against 0.8)
-  D.staging_bytes = (size_t)std::max(D.staging_slots * slot_bytes, std::min(kStagingBytes, state));
-  D.staging = reinterpret_cast<float *>(k.take<uint8_t>(D.staging_bytes));
+  *staging_bytes = (size_t)std::max(D.staging_slots * slot_bytes, std::min(kStagingBytes, state));
+  D.staging = reinterpret_cast<float *>(k.take<uint8_t>(*staging_bytes));
   // The policy kernel's FP8 tail batches and its requests into L1 reach up
   // to kStreamSlack bytes past the last weight block (no product uses them):
   // the regions after the weights (the histogram alone is 256 KB per world)
@@ -374,7 +378,8 @@ extern "C" int eco_workspace_bytes(const eco_config *cfg, size_t *bytes) {
   Layout L = make_layout(cfg);
   Dev d;
   EnvDesc *ed;
-  *bytes = carve(cfg, L, nullptr, &d, &ed);
+  size_t staging;
+  *bytes = carve(cfg, L, nullptr, &d, &ed, &staging);
   return ECO_OK;
 }
 
@@ -455,7 +460,7 @@ extern "C" int eco_create(const eco_config *cfg, void *dev_workspace, size_t byt
   R.res_cap = cfg->res_cap;
   h->ws = reinterpret_cast<uint8_t *>(dev_workspace);
   h->ws_bytes = bytes;
-  carve(cfg, h->L, h->ws, &h->d, &h->env_dev);
+  carve(cfg, h->L, h->ws, &h->d, &h->env_dev, &h->staging_bytes);
   int so = 0, co = 0, to = 0;
   for (int e = 0; e < cfg->n_envs; ++e) {
     EnvDesc ed;
@@ -1036,7 +1041,7 @@ extern "C" int eco_read_state(eco_handle *h, int32_t env, eco_state_view *out) {
                {out->photo, d.photo + co, 4 * N},    {out->step, d.step, sizeof(int64_t)}};
   // arrays a kernel converts: every cell's food, wall and env-local occupant
   // (6 bytes a cell), every slot's x, y and RGB (20 bytes a slot)
-  const size_t staging = d.staging_bytes;
+  const size_t staging = h->staging_bytes;
   if (state_bytes(N, S) <= kBounceBytes) {
     // a small world: everything packed by one kernel and brought over by one
     // copy into pinned memory (a copy per array cost 0.3 ms)

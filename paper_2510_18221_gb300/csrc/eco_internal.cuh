@@ -308,11 +308,10 @@ struct Dev {
   int32_t *place_tiles;     // [place_tile_count] founders per placement tile
   int place_tile_count;
   uint8_t *bflag;          // [total_slots] birth pass flags
-  float *staging;          // staging_bytes: parameters in logical order (of staging_slots
-                           // slots at a time) or a state's converted arrays, on their way
-                           // between the host and the device's arrays
+  float *staging;          // parameters in logical order (of staging_slots slots at a time)
+                           // or a state's converted arrays, on their way between the host
+                           // and the device's arrays
   int staging_slots;
-  size_t staging_bytes;
   int32_t *hp;             // [total_slots] paper rules: HP (quarter points)
   int32_t *age;            // [total_slots] paper rules: steps survived
   int32_t *res;            // [total_cells] paper rules: energy on the cell
