@@ -22,6 +22,10 @@
  *     eco_workspace_bytes() reports, 256-byte aligned, and keeps it alive
  *     until eco_destroy().  The library carves every device array out of
  *     it, allocates no other device memory, and never frees caller memory.
+ *     The size is this build's: a stored one from another build may be too
+ *     small (ECO_ENOMEM).  It includes a staging region of at most 32 MB
+ *     (more only where one slot's parameters are more) through which states
+ *     and parameters cross between the host and the device's layout.
  *     Each handle holds three small pinned host buffers for the statistics
  *     and status word (about 2 x n_envs x 8 x ECO_N_STATS bytes each; one
  *     for eco_read_stats(), two for eco_step_read()) and, when one of its
@@ -33,6 +37,9 @@
  *     and eco_write_*() synchronise that stream.
  *   - Host buffers passed to eco_read_* / eco_write_* are caller-owned,
  *     sized as documented per function, and are not retained.
+ *     eco_read_state, eco_read_params and eco_write_params of one handle may
+ *     be called by several host threads (they take turns); handles are
+ *     independent of one another.
  *   - Environments are independent: environment e, run alone or batched
  *     with others, produces identical results.
  */
@@ -188,9 +195,9 @@ typedef struct {
                                     the order of FP32 additions); k > 0 =
                                     force variant k (eco_policy_variants) */
   int32_t launch_mode;           /* environment phases: 0 = one persistent
-                                    cooperative kernel when the device
-                                    supports it, 1 = one kernel per phase
-                                    (identical results)                     */
+                                    kernel when the device supports it,
+                                    1 = one kernel per phase (identical
+                                    results)                                */
   int32_t policy_form;           /* ECO_POLICY_PLAIN or ECO_POLICY_PAPER     */
   int32_t n_hidden;              /* paper form: hidden H -> H layers (1..4);
                                     the plain form ignores it (one layer)   */
@@ -346,10 +353,11 @@ int eco_reset_seed(eco_handle *h, uint64_t seed);
  * ECO_ETIMEOUT by the next eco_read_stats(). */
 int eco_step(eco_handle *h, int32_t n_steps);
 
-/* Pipelined step and read: enqueue one step whose graph ends by copying
- * the statistics and status word into one of two pinned buffers the handle
- * owns, then wait for the copy made by the PREVIOUS eco_step_read call and
- * return those records.  So a call returns the records as of the end of
+/* Pipelined step and read: enqueue one step that leaves its statistics and
+ * status word in one of two pinned buffers the handle owns (the environment
+ * kernel stores them; the one-kernel-per-phase form ends with a copy), then
+ * wait for the step of the PREVIOUS eco_step_read call and return its
+ * records.  So a call returns the records as of the end of
  * the step enqueued by the previous call (on the first call after
  * eco_create or eco_reset: the records as they stood when the call was
  * made), while the step it enqueued runs; eco_read_stats afterwards gives
@@ -421,14 +429,18 @@ int eco_read_streamed_bias(eco_handle *h, int32_t env, int32_t slot0, int32_t n,
 int eco_read_policy_io(eco_handle *h, int32_t env, float *logits, uint8_t *actions);
 
 /* Policy-kernel variants: *count variants exist; *chosen is the one in use.
- * eco_policy_variant_name() describes variant k (static string). */
+ * eco_policy_variant_name() describes variant k (static string); what a
+ * number stands for is this build's, the results of all dense variants are
+ * the same. */
 int eco_policy_variants(const eco_handle *h, int32_t *count, int32_t *chosen);
 const char *eco_policy_variant_name(int32_t k);
 
 /* Launch form of the environment phases in use: *mode 0 = one persistent
- * cooperative kernel of *blocks CTAs, 1 = one kernel per phase.  Decided at
- * the first eco_step (falls back to 1 when the device or the graph capture
- * does not support the cooperative form). */
+ * kernel of *blocks CTAs -- a cooperative launch whose phases are separated
+ * by bounded grid barriers or, for a batch of at most 4,096 slots and 16,384
+ * cells, one cluster of 8 CTAs with the hardware's cluster barrier -- 1 = one
+ * kernel per phase.  Decided at the first eco_step (falls back to 1 when the
+ * device or the graph capture does not support the persistent form). */
 int eco_launch_mode(const eco_handle *h, int32_t *mode, int32_t *blocks);
 
 /* Like eco_step, and also times policy-kernel launches with a CUDA-event
@@ -447,12 +459,13 @@ int eco_policy_timing(eco_handle *h, double *total_ms, int32_t *n_timed, int64_t
 
 /* Run only the policy phase (observe + MLP + sample) of the current state
  * n_iters times, for timing and for the policy-parity tests; the world
- * state does not change.  Asynchronous. */
+ * state does not change.  (Behind steps that no eco_read_stats has found
+ * complete, the list of alive agents is made again first.)  Asynchronous. */
 int eco_policy_only(eco_handle *h, int32_t n_iters);
 
 /* Failure-detection test hook (off unless called; cleared by eco_reset).
- * The persistent environment kernel separates its phases with grid
- * barriers whose waits are bounded; this arms the next steps so that CTA
+ * The persistent environment kernel's cooperative form separates its phases
+ * with grid barriers whose waits are bounded; this arms the next steps so that CTA
  * absent_cta leaves that kernel before its first barrier and every wait
  * gives up after poll_budget polls (a few ms for 10^5).  The other CTAs'
  * waits then run out: the status word records the timeout, every CTA
@@ -460,9 +473,10 @@ int eco_policy_only(eco_handle *h, int32_t n_iters);
  * once, and the next eco_read_stats / eco_step_read returns ECO_ETIMEOUT.
  * The world state is then partly stepped; eco_reset (or eco_reset_seed)
  * clears the barrier, the status word and these test words.  ECO_EINVAL
- * when the persistent form with more than one CTA is not in use
- * (eco_launch_mode; it is decided at the first eco_step) or for an
- * argument out of range.  Synchronises. */
+ * when that form is not in use (eco_launch_mode; it is decided at the first
+ * eco_step) or for an argument out of range.  A small batch's cluster waits
+ * at hardware barriers, which no CTA can miss and which have no budget: it
+ * cannot be armed and never times out.  Synchronises. */
 int eco_arm_barrier_timeout(eco_handle *h, int32_t absent_cta, int32_t poll_budget);
 
 /* Phase trace of the persistent environment kernel (a tracing aid; App. E

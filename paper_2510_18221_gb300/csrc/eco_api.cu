@@ -526,7 +526,8 @@ extern "C" int eco_create(const eco_config *cfg, void *dev_workspace, size_t byt
   if (e == cudaSuccess && h->grid.persistent_blocks > 0) {
     // a batch of at most 4,096 slots and 16,384 cells runs the persistent
     // form on one cluster of eight CTAs, whose barriers are the hardware's
-    // (0.3 us against 1.1) while its births still spread over 8,192 threads;
+    // (0.5-0.6 us from the last arrival to CTA 0's pass by the phase trace,
+    // against 1.1) while its births still spread over 8,192 threads;
     // anything larger keeps one CTA per SM
     const long long work = std::max((long long)h->d.total_slots, (long long)h->d.total_cells / 4);
     if (work <= 4096) env_use_small_grid(h->L, &h->grid);
@@ -997,8 +998,10 @@ extern "C" int eco_step_read(eco_handle *h, eco_stats *total, eco_stats *last, i
 }
 
 // ---------------------------------------------------------------------------
-// State and parameter I/O (host-side marshalling between the library's
-// layout and the plain views of the header).
+// State and parameter I/O.  Reads and eco_write_params convert between the
+// library's layout and the plain views of the header on the device, in the
+// workspace's staging region; eco_write_state and the streamed copy's readers
+// marshal on the host.
 // ---------------------------------------------------------------------------
 
 static int check_env(eco_handle *h, int32_t env) {

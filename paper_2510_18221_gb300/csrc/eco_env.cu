@@ -3,23 +3,28 @@
 // of the batch at once.
 //
 // Phase order: policy (+ facing, turns and move claims, fused into its
-// epilogue; eco_policy.cu) -> move apply + eat + attack claims on cells ->
-// attack transfers + metabolism + death -> birth claims (+ regrowth, which
-// commutes with them) -> slot assignment -> mutation of the children, the
-// alive list of the next step and the statistics.
+// epilogue; eco_policy_kernel.cuh) -> move apply + eat + attack claims on
+// cells -> attack transfers + metabolism + death (+ regrowth under the simple
+// rules, where only eating takes food) -> birth claims (+ regrowth under the
+// other rules, which commutes with them) -> slot assignment -> mutation of
+// the children, the alive list of the next step and the statistics.
 //
-// Two launch forms run the same phase functions: one persistent kernel
-// (cooperative launch; phases separated by grid barriers whose waits are
-// bounded, so a stuck barrier sets the status word and every CTA exits), and
-// one kernel per phase.  Both give bit-identical results.
+// Two launch forms run the same phase functions: one persistent kernel and
+// one kernel per phase.  Both give bit-identical results.  The persistent
+// kernel is a cooperative launch whose phases are separated by grid barriers
+// with bounded waits (a stuck barrier sets the status word and every CTA
+// exits) or, for a small batch, one thread-block cluster, whose hardware
+// barrier needs no bound: its CTAs are resident together.
 //
 // Conflicts (two movers into one free cell, two attackers on one victim's
 // cell, two parents onto one birth cell) are resolved by a 64-bit atomicMax
 // of (Philox draw << 32 | ~local slot): the highest draw wins, equal draws
 // go to the lower slot.  A maximum does not depend on the order of the
-// atomics, every other atomic is an integer add, and no phase's result
-// depends on the order in which agents are visited, so all integer state
-// is bit-identical from run to run and equal to the plain sequential rule.
+// atomics; the others are integer adds and, where deaths and regrowth share
+// an interval, ands and ors of different bits of a cell's word; and no
+// phase's result depends on the order in which agents are visited, so all
+// integer state is bit-identical from run to run and equal to the plain
+// sequential rule.
 #include "eco_internal.cuh"
 #include "eco_kernels.h"
 
@@ -1524,7 +1529,7 @@ __global__ void __launch_bounds__(1024) k_finish(Dev d, Rules R) {
 #undef STEP_T
 
 // ---------------------------------------------------------------------------
-// The persistent form: all phases in one cooperative launch.
+// The persistent form: all phases in one launch.
 // ---------------------------------------------------------------------------
 constexpr unsigned kBarrierSpinLimit = 40u * 1000u * 1000u;  // x >= 64 ns: > 2.5 s
 constexpr int kStatusTimeout = 4;
@@ -1681,7 +1686,9 @@ __device__ __forceinline__ unsigned long long global_ns() {
 }
 
 // CLUSTER: the grid is one thread-block cluster, whose hardware barrier takes
-// the grid barrier's place.
+// the grid barrier's place.  1,024 threads leave 64 registers each, and 32
+// bytes are spilled (48 reloaded) at that cap: the agents' words and the
+// regrowth's draws are kept in registers across the phases.
 template <bool CLUSTER>
 __global__ void __launch_bounds__(1024, 1) k_env_persistent(Dev d, Layout L, Rules R) {
   extern __shared__ __align__(16) float msm[];

@@ -86,10 +86,11 @@ __global__ void k_na_apply(const unsigned long long *claims, int side, int n, co
 // cluster of kClusterCtas CTAs, whose hardware barrier separates clearing,
 // claiming and applying, with up to kPerThread agents' targets kept in
 // registers.  Only the cells that are claimed are cleared.  Bound by three
-// round trips and the launch: a caller's calls for 300 agents take 8.9 us
-// each and for 12,000 agents 9.9, in place of 13.4 with three launches, whose
-// issue bounds them; at 32,000 agents on eight SMs (12.3 us, and a single
-// call alone 1 us longer) the gain is gone, and the three launches stay.
+// round trips and the launch.  us per call on a stream of their own, called
+// from Python back to back (each waited for), three launches -> one: 300
+// agents 12.3 -> 6.1 (21.4 -> 15.3), 12,000 12.3 -> 9.4 (21.6 -> 18.3), 16,384
+// 12.3 -> 10.2 (21.7 -> 18.5).  At 32,000 agents on eight SMs the gain is gone
+// (12.3 us, and a single call alone 1 us longer), and the three launches stay.
 constexpr int kClusterCtas = 8;
 constexpr int kClusterThreads = 1024;
 constexpr int kPerThread = 2;
