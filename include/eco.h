@@ -22,8 +22,8 @@
  *     eco_workspace_bytes() reports, 256-byte aligned, and keeps it alive
  *     until eco_destroy().  The library carves every device array out of
  *     it, allocates no other device memory, and never frees caller memory.
- *     The size is this build's: a stored one from another build may be too
- *     small (ECO_ENOMEM).  It includes a staging region of at most 32 MB
+ *     The size is that of the library in use: one stored with another
+ *     version may be too small (ECO_ENOMEM).  It includes a staging region of at most 32 MB
  *     (more only where one slot's parameters are more) through which states
  *     and parameters cross between the host and the device's layout.
  *     Each handle holds three small pinned host buffers for the statistics
@@ -430,8 +430,8 @@ int eco_read_policy_io(eco_handle *h, int32_t env, float *logits, uint8_t *actio
 
 /* Policy-kernel variants: *count variants exist; *chosen is the one in use.
  * eco_policy_variant_name() describes variant k (static string); what a
- * number stands for is this build's, the results of all dense variants are
- * the same. */
+ * number stands for may change with the library's version, the results of
+ * all dense variants are the same. */
 int eco_policy_variants(const eco_handle *h, int32_t *count, int32_t *chosen);
 const char *eco_policy_variant_name(int32_t k);
 
